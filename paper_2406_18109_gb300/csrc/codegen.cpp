@@ -24,6 +24,7 @@
 #include <functional>
 #include <sstream>
 #include <stdexcept>
+#include <tuple>
 
 #include "runtime.hpp"
 
@@ -123,6 +124,7 @@ class Gen {
   int nbar = 0;
   int nbc = 0;  // shared broadcast slots of finished reductions
   bool stage = false;  // some per-point SpMV nest stages x windows in shared memory
+  int wave_blocks = 0;  // CTAs per SM an in-place sweep needs resident
 
   const LaunchRoot& R(int64_t root) const { return S.roots[S.root_index.at(root)]; }
   bool temp_in(int g, int64_t root) const;
@@ -134,7 +136,29 @@ class Gen {
   void emit_group(int g);
   void emit_scalar_group(int g);
   void emit_vector_group(int g);
+  // memory reads of a loop nest: distinct (root, partition) read before any
+  // in-nest write of it; reduction accumulators
+  struct Rd { std::string key; const Arg* a; std::string var; bool ro; };
+  struct Acc { int task; int slot; std::string var; int dt; };
+  // What the body of a nest needs besides its loads: names of the base
+  // offsets and immediates, SpMV values computed before the body, the SpMV
+  // task that reads staged x windows.
+  struct BodyEnv {
+    std::vector<Rd> reads;
+    std::vector<Acc> accs;
+    std::map<std::string, std::string> base;
+    std::map<std::pair<int, int>, std::string> immv;
+    std::map<int, std::string> spre;
+    int staged = -1;
+  };
   void emit_nest(int g, const Nest& n, const std::string& red_pt, bool flat);
+  std::map<std::string, std::vector<std::string>> emit_compute(const Nest& n, const BodyEnv& E, int w,
+                                                               const std::vector<std::string>& slots,
+                                                               const std::vector<std::string>& eflat,
+                                                               const std::string& pad);
+  void emit_wave(int g);
+  void emit_march(int g, int sweeps);
+  std::string sweep_signature(int g) const;
   // Which tasks of nest n run two lanes per instruction in a body of w lanes
   // (index: task - n.first).
   std::vector<char> packed_tasks(const Nest& n, int w) const;
@@ -467,6 +491,146 @@ std::vector<char> Gen::packed_tasks(const Nest& n, int w) const {
   return pk;
 }
 
+// The tasks of a nest over `slots` groups of w lanes, in program order, on
+// values the caller has loaded as <read var>_<slot>.  Returns, per (root,
+// partition) to store, the value names by slot * w + lane.
+std::map<std::string, std::vector<std::string>> Gen::emit_compute(const Nest& n, const BodyEnv& E, int w,
+                                                                  const std::vector<std::string>& slots,
+                                                                  const std::vector<std::string>& eflat,
+                                                                  const std::string& pad) {
+  const int ns = (int)slots.size();
+  // compute: per slot, tasks in program order, each over the lanes
+  const std::vector<char> pk = packed_tasks(n, w);
+  std::map<std::string, std::vector<std::string>> outvars;  // akey -> per (slot*w+lane) value
+  for (int s = 0; s < ns; ++s) {
+    std::vector<std::map<std::string, std::string>> curs(w);  // per lane: akey -> value expr
+    std::vector<LaneOps> lanes(w);
+    for (int l = 0; l < w; ++l)
+      for (const Rd& rd : E.reads) {
+        const std::string v = rd.var + "_" + slots[s];
+        curs[l][rd.key] = (w > 1) ? v + ".v[" + std::to_string(l) + "]" : v;
+      }
+    for (int i = n.first; i < n.last; ++i) {
+      const Task& t = S.tasks[i];
+      if (t.scalar()) continue;
+      const int dt = space_arg(t).dtype;   // the output's (y for an SpMV, whose last arg may be its windows)
+      auto res_of = [&](int l) { return "v" + std::to_string(i) + "_" + slots[s] + "_" + std::to_string(l); };
+      auto val_of = [&](int l, size_t ai) -> std::string {
+        const Arg& a = t.args[ai];
+        if (a.imm) return E.immv.at({i, (int)ai});
+        if (a.nd == 0) return "(" + T(dt) + ")" + sreg.at(a.root);
+        return curs[l].at(akey(a));
+      };
+      if (pk[i - n.first]) {
+        // two lanes per instruction
+        for (int l = 0; l < w; l += 2) {
+          const std::string r0 = res_of(l), r1 = res_of(l + 1), pr = r0 + "_p";
+          if (t.op == DFS_OP_NCDF || t.op == DFS_OP_ERF) {
+            lanes[l].define(r0);
+            lanes[l + 1].define(r1);
+            const std::string a0 = val_of(l, 0), a1 = val_of(l + 1, 0);
+            // the argument of erf: x / sqrt 2 for NCDF, x itself for ERF
+            std::string y0 = a0, y1 = a1;
+            if (t.op == DFS_OP_NCDF) {
+              const std::string y = r0 + "_y2";
+              o << pad << "const float2 " << y << " = pk_ncdf_arg(" << a0 << ", " << a1 << ");\n";
+              y0 = y + ".x";
+              y1 = y + ".y";
+            }
+            // erf(|y|) of both lanes in one packed evaluation, unless the
+            // lanes reuse the magnitude of a negation (both do, or neither)
+            std::string m0 = lanes[l].mag_of(t.op, a0), m1 = lanes[l + 1].mag_of(t.op, a1);
+            if (m0.empty() && m1.empty()) {
+              o << pad << "const float2 " << r0 << "_m2 = erf_mag2(" << y0 << ", " << y1 << ");\n";
+              m0 = r0 + "_m2.x";
+              m1 = r0 + "_m2.y";
+            } else {
+              if (m0.empty()) {
+                m0 = r0 + "_m";
+                o << pad << "const float " << m0 << " = erf_mag(" << y0 << ");\n";
+              }
+              if (m1.empty()) {
+                m1 = r1 + "_m";
+                o << pad << "const float " << m1 << " = erf_mag(" << y1 << ");\n";
+              }
+            }
+            lanes[l].set_mag(t.op, a0, m0);
+            lanes[l + 1].set_mag(t.op, a1, m1);
+            if (t.op == DFS_OP_NCDF)
+              o << pad << "const float2 " << pr << " = pk_ncdf_of_erf(erf_sign(" << m0 << ", " << y0 << "), erf_sign("
+                << m1 << ", " << y1 << "));\n";
+            else
+              o << pad << "const float2 " << pr << " = make_float2(erf_sign(" << m0 << ", " << y0 << "), erf_sign("
+                << m1 << ", " << y1 << "));\n";
+          } else if (t.op == DFS_OP_LOG) {
+            lanes[l].define(r0);
+            lanes[l + 1].define(r1);
+            o << pad << "const float2 " << pr << " = log_f32x2(" << val_of(l, 0) << ", " << val_of(l + 1, 0) << ");\n";
+          } else {
+            lanes[l].define(r0);
+            lanes[l + 1].define(r1);
+            o << pad << "const float2 " << pr << " = pk_add(" << val_of(l, 0) << ", " << val_of(l + 1, 0) << ", "
+              << val_of(l, 1) << ", " << val_of(l + 1, 1) << ");\n";
+          }
+          o << pad << "const float " << r0 << " = " << pr << ".x;\n";
+          o << pad << "const float " << r1 << " = " << pr << ".y;\n";
+          curs[l][akey(t.args.back())] = r0;
+          curs[l + 1][akey(t.args.back())] = r1;
+        }
+        continue;
+      }
+      for (int l = 0; l < w; ++l) {
+        auto& cur = curs[l];
+        LaneOps& lane = lanes[l];
+        auto val = [&](size_t ai) { return val_of(l, ai); };
+        const std::string res = res_of(l);
+        if (is_elementwise(t.op)) {
+          std::vector<std::string> in{val(0)};
+          if (t.args.size() == 3) in.push_back(val(1));
+          lane.emit(o, pad, T(dt), t.op, res, in);
+          cur[akey(t.args.back())] = res;
+        } else if (t.op == DFS_OP_SPMV && E.spre.count(i)) {
+          o << pad << "const " << T(dt) << " " << res << " = " << E.spre.at(i) << "_" << l << ";\n";
+          cur[akey(t.args[4])] = res;
+        } else if (t.op == DFS_OP_SPMV) {
+          const Arg& y = t.args[4];
+          const std::string row = "(" + E.base.at(akey(y)) + " - " + std::to_string(y.part.vlo[0]) + "LL + " +
+                                  eflat[s] + " + " + std::to_string(l) + ")";
+          o << pad << "const " << T(dt) << " " << res << " = " << (i == E.staged ? "spmv_row_xs<" : "spmv_row<")
+            << T(dt) << ">(" << ptr(t.args[0].root) << " + " << E.base.at(akey(t.args[0])) << ", "
+            << ptr(t.args[1].root) << " + " << E.base.at(akey(t.args[1])) << ", " << ptr(t.args[2].root) << " + "
+            << E.base.at(akey(t.args[2])) << ", " << ptr(t.args[3].root) << " + " << E.base.at(akey(t.args[3])) << ", "
+            << row << (i == E.staged ? ", (const " + T(dt) + "*)dfs_xs_raw, xw_" : std::string()) << ");\n";
+          cur[akey(y)] = res;
+        } else if (is_reduction(t.op)) {
+          const Acc* ac = nullptr;
+          for (const Acc& x : E.accs)
+            if (x.task == i) ac = &x;
+          if (t.op == DFS_OP_DOT)
+            o << pad << ac->var << " = red_fma(" << val(0) << ", " << val(1) << ", " << ac->var << ");\n";
+          else
+            o << pad << ac->var << " = " << ac->var << " + " << val(0) << ";\n";
+        }
+      }
+    }
+    // collect outputs to store
+    for (int l = 0; l < w; ++l)
+      for (int i = n.first; i < n.last; ++i) {
+        const Task& t = S.tasks[i];
+        if (t.scalar()) continue;
+        const Arg* out = nullptr;
+        if (is_elementwise(t.op)) out = &t.args.back();
+        if (t.op == DFS_OP_SPMV) out = &t.args[4];
+        if (!out || R(out->root).temp) continue;
+        const std::string k = akey(*out);
+        auto& vv = outvars[k];
+        if (vv.size() < (size_t)(ns * w)) vv.resize(ns * w);
+        vv[s * w + l] = curs[l].at(k);
+      }
+  }
+  return outvars;
+}
+
 void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
   const int BD = S.block;
   const int U = std::max(1, S.unroll);
@@ -478,7 +642,8 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
   o << ind << "{ // nest: tasks " << n.first << ".." << n.last - 1 << ", vec " << V << ", "
     << (n.dims == 1 ? "flat" : "rows") << "\n";
   // ---- per-access base offsets (root coordinates flattened)
-  std::map<std::string, std::string> base;  // akey -> base variable
+  BodyEnv E;
+  std::map<std::string, std::string>& base = E.base;  // akey -> base variable
   int nb = 0;
   auto box_lo = [&](const Arg& a, int d) {
     std::ostringstream s;
@@ -525,13 +690,10 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
   }
   // ---- classify accesses
   // reads from memory: distinct (root, partition) read before any in-nest write of it
-  struct Rd { std::string key; const Arg* a; std::string var; bool ro; };
-  std::vector<Rd> reads;
+  std::vector<Rd>& reads = E.reads;
   std::map<std::string, int> read_idx;
   std::set<std::string> written_keys;
-  // reduction accumulators
-  struct Acc { int task; int slot; std::string var; int dt; };
-  std::vector<Acc> accs;
+  std::vector<Acc>& accs = E.accs;  // reduction accumulators
   for (int i = n.first; i < n.last; ++i) {
     const Task& t = S.tasks[i];
     if (t.scalar()) continue;
@@ -577,7 +739,7 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
   }
   // the first SpMV of a per-point nest that carries x windows: stage them for
   // this point (every thread of the CTA is here, at the same point)
-  int staged = -1;
+  int& staged = E.staged;
   if (stage && !flat && n.dims == 1 && !n.coop)
     for (int i = n.first; i < n.last && staged < 0; ++i)
       if (S.tasks[i].op == DFS_OP_SPMV && S.tasks[i].args.size() == 6) staged = i;
@@ -592,7 +754,7 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
       << ", &xs_mbar_, xs_ph_, xs_live_, ctl, P.timeout_ns);\n";
   }
   // immediates hoisted once per nest
-  std::map<std::pair<int, int>, std::string> immv;
+  std::map<std::pair<int, int>, std::string>& immv = E.immv;
   for (int i = n.first; i < n.last; ++i) {
     const Task& t = S.tasks[i];
     if (t.scalar()) continue;
@@ -606,7 +768,7 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
     }
   }
 
-  std::map<int, std::string> spre;  // SpMV task -> value computed before the body (warp-cooperative rows)
+  std::map<int, std::string>& spre = E.spre;  // SpMV task -> value computed before the body (warp-cooperative rows)
   // ---- body generator for one element group: `u` unroll slot, lanes V,
   // element offset expression `eoff` (flat) or (row, col) expressions
   auto addr = [&](const Arg& a, const std::string& e_flat, const std::string& row, const std::string& col) {
@@ -644,135 +806,7 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
         }
       }
     }
-    // compute: per slot, tasks in program order, each over the lanes
-    const std::vector<char> pk = packed_tasks(n, w);
-    std::map<std::string, std::vector<std::string>> outvars;  // akey -> per (slot*w+lane) value
-    for (int s = 0; s < ns; ++s) {
-      std::vector<std::map<std::string, std::string>> curs(w);  // per lane: akey -> value expr
-      std::vector<LaneOps> lanes(w);
-      for (int l = 0; l < w; ++l)
-        for (const Rd& rd : reads) {
-          const std::string v = rd.var + "_" + slots[s];
-          curs[l][rd.key] = (w > 1) ? v + ".v[" + std::to_string(l) + "]" : v;
-        }
-      for (int i = n.first; i < n.last; ++i) {
-        const Task& t = S.tasks[i];
-        if (t.scalar()) continue;
-        const int dt = space_arg(t).dtype;   // the output's (y for an SpMV, whose last arg may be its windows)
-        auto res_of = [&](int l) { return "v" + std::to_string(i) + "_" + slots[s] + "_" + std::to_string(l); };
-        auto val_of = [&](int l, size_t ai) -> std::string {
-          const Arg& a = t.args[ai];
-          if (a.imm) return immv.at({i, (int)ai});
-          if (a.nd == 0) return "(" + T(dt) + ")" + sreg.at(a.root);
-          return curs[l].at(akey(a));
-        };
-        if (pk[i - n.first]) {
-          // two lanes per instruction
-          for (int l = 0; l < w; l += 2) {
-            const std::string r0 = res_of(l), r1 = res_of(l + 1), pr = r0 + "_p";
-            if (t.op == DFS_OP_NCDF || t.op == DFS_OP_ERF) {
-              lanes[l].define(r0);
-              lanes[l + 1].define(r1);
-              const std::string a0 = val_of(l, 0), a1 = val_of(l + 1, 0);
-              // the argument of erf: x / sqrt 2 for NCDF, x itself for ERF
-              std::string y0 = a0, y1 = a1;
-              if (t.op == DFS_OP_NCDF) {
-                const std::string y = r0 + "_y2";
-                o << pad << "const float2 " << y << " = pk_ncdf_arg(" << a0 << ", " << a1 << ");\n";
-                y0 = y + ".x";
-                y1 = y + ".y";
-              }
-              // erf(|y|) of both lanes in one packed evaluation, unless the
-              // lanes reuse the magnitude of a negation (both do, or neither)
-              std::string m0 = lanes[l].mag_of(t.op, a0), m1 = lanes[l + 1].mag_of(t.op, a1);
-              if (m0.empty() && m1.empty()) {
-                o << pad << "const float2 " << r0 << "_m2 = erf_mag2(" << y0 << ", " << y1 << ");\n";
-                m0 = r0 + "_m2.x";
-                m1 = r0 + "_m2.y";
-              } else {
-                if (m0.empty()) {
-                  m0 = r0 + "_m";
-                  o << pad << "const float " << m0 << " = erf_mag(" << y0 << ");\n";
-                }
-                if (m1.empty()) {
-                  m1 = r1 + "_m";
-                  o << pad << "const float " << m1 << " = erf_mag(" << y1 << ");\n";
-                }
-              }
-              lanes[l].set_mag(t.op, a0, m0);
-              lanes[l + 1].set_mag(t.op, a1, m1);
-              if (t.op == DFS_OP_NCDF)
-                o << pad << "const float2 " << pr << " = pk_ncdf_of_erf(erf_sign(" << m0 << ", " << y0 << "), erf_sign("
-                  << m1 << ", " << y1 << "));\n";
-              else
-                o << pad << "const float2 " << pr << " = make_float2(erf_sign(" << m0 << ", " << y0 << "), erf_sign("
-                  << m1 << ", " << y1 << "));\n";
-            } else if (t.op == DFS_OP_LOG) {
-              lanes[l].define(r0);
-              lanes[l + 1].define(r1);
-              o << pad << "const float2 " << pr << " = log_f32x2(" << val_of(l, 0) << ", " << val_of(l + 1, 0) << ");\n";
-            } else {
-              lanes[l].define(r0);
-              lanes[l + 1].define(r1);
-              o << pad << "const float2 " << pr << " = pk_add(" << val_of(l, 0) << ", " << val_of(l + 1, 0) << ", "
-                << val_of(l, 1) << ", " << val_of(l + 1, 1) << ");\n";
-            }
-            o << pad << "const float " << r0 << " = " << pr << ".x;\n";
-            o << pad << "const float " << r1 << " = " << pr << ".y;\n";
-            curs[l][akey(t.args.back())] = r0;
-            curs[l + 1][akey(t.args.back())] = r1;
-          }
-          continue;
-        }
-        for (int l = 0; l < w; ++l) {
-          auto& cur = curs[l];
-          LaneOps& lane = lanes[l];
-          auto val = [&](size_t ai) { return val_of(l, ai); };
-          const std::string res = res_of(l);
-          if (is_elementwise(t.op)) {
-            std::vector<std::string> in{val(0)};
-            if (t.args.size() == 3) in.push_back(val(1));
-            lane.emit(o, pad, T(dt), t.op, res, in);
-            cur[akey(t.args.back())] = res;
-          } else if (t.op == DFS_OP_SPMV && spre.count(i)) {
-            o << pad << "const " << T(dt) << " " << res << " = " << spre.at(i) << "_" << l << ";\n";
-            cur[akey(t.args[4])] = res;
-          } else if (t.op == DFS_OP_SPMV) {
-            const Arg& y = t.args[4];
-            const std::string row = "(" + base.at(akey(y)) + " - " + std::to_string(y.part.vlo[0]) + "LL + " +
-                                    eflat[s] + " + " + std::to_string(l) + ")";
-            o << pad << "const " << T(dt) << " " << res << " = " << (i == staged ? "spmv_row_xs<" : "spmv_row<")
-              << T(dt) << ">(" << ptr(t.args[0].root) << " + " << base.at(akey(t.args[0])) << ", "
-              << ptr(t.args[1].root) << " + " << base.at(akey(t.args[1])) << ", " << ptr(t.args[2].root) << " + "
-              << base.at(akey(t.args[2])) << ", " << ptr(t.args[3].root) << " + " << base.at(akey(t.args[3])) << ", "
-              << row << (i == staged ? ", (const " + T(dt) + "*)dfs_xs_raw, xw_" : std::string()) << ");\n";
-            cur[akey(y)] = res;
-          } else if (is_reduction(t.op)) {
-            const Acc* ac = nullptr;
-            for (const Acc& x : accs)
-              if (x.task == i) ac = &x;
-            if (t.op == DFS_OP_DOT)
-              o << pad << ac->var << " = red_fma(" << val(0) << ", " << val(1) << ", " << ac->var << ");\n";
-            else
-              o << pad << ac->var << " = " << ac->var << " + " << val(0) << ";\n";
-          }
-        }
-      }
-      // collect outputs to store
-      for (int l = 0; l < w; ++l)
-        for (int i = n.first; i < n.last; ++i) {
-          const Task& t = S.tasks[i];
-          if (t.scalar()) continue;
-          const Arg* out = nullptr;
-          if (is_elementwise(t.op)) out = &t.args.back();
-          if (t.op == DFS_OP_SPMV) out = &t.args[4];
-          if (!out || R(out->root).temp) continue;
-          const std::string k = akey(*out);
-          auto& vv = outvars[k];
-          if (vv.size() < (size_t)(ns * w)) vv.resize(ns * w);
-          vv[s * w + l] = curs[l].at(k);
-        }
-    }
+    const auto outvars = emit_compute(n, E, w, slots, eflat, pad);
     // stores (the last value written to each (root, partition) in the nest)
     for (auto& kv : outvars) {
       const Arg* a = nullptr;
@@ -1056,6 +1090,736 @@ int Gen::emit_warp0_scalars(int g) {
   return h;
 }
 
+// ------------------------------------------------------- in-place sweeps
+// See WaveGeom and MarchGeom.  The two-phase form of a Fig. 1 sweep (the
+// stencil into a second array, a grid barrier, the copy back) moves 16 bytes
+// per FP32 point and is bound by HBM; in place it is 8.  Measured on GB300, us
+// per sweep, two phases -> in place:
+//   8190^2 FP32 (512-thread CTAs)        175.6 -> 91.9 (5.84 TB/s, 86 % of the copy rate)
+//   1021 x 1147 FP32, five per launch      8.3 -> 4.4
+//   4000^2 FP64                          197.4 -> 174.4 (bound by the FP64 pipe: 5 operations per point)
+//   251^3 FP32 (tiles)                    64.1 -> 42.1
+//   251^3 FP64 (tiles)                   258.9 -> 242 (FP64 pipe: 7 operations per point, 176 us)
+int64_t origin_of(const Arg& a, int d) { return std::max(a.part.off[d], a.part.vlo[d]); }
+int64_t floor_div(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
+
+}  // namespace
+
+bool wave_legal(const LaunchSpec& S, int g) {
+  if (g + 1 >= (int)S.groups.size()) return false;
+  const Group &A = S.groups[g], &B = S.groups[g + 1];
+  if (A.scalar || B.scalar) return false;
+  const std::string space = iteration_space_key(S.tasks[A.begin]);
+  for (int i = A.begin; i < B.end; ++i) {
+    const Task& t = S.tasks[i];
+    if (t.scalar() || !is_elementwise(t.op) || iteration_space_key(t) != space) return false;
+    for (const Arg& a : t.args) {
+      if (a.imm || a.nd == 0) continue;
+      if (a.nd != 2 && a.nd != 3) return false;
+      if (a.part.kind != 1) return false;
+      for (int d = 0; d < a.nd; ++d)
+        if (a.part.proj[d] != d) return false;
+    }
+  }
+  // across the groups, accesses of one store through different partitions may
+  // only be a read in A and a write in B (the anti-dependence the wave orders)
+  bool cut = false;
+  for (int i = A.begin; i < A.end; ++i)
+    for (const Arg& a : S.tasks[i].args) {
+      if (a.imm || a.nd == 0) continue;
+      for (int j = B.begin; j < B.end; ++j)
+        for (const Arg& b : S.tasks[j].args) {
+          if (b.imm || b.root != a.root || b.part == a.part) continue;
+          if (a.is_w()) return false;
+          if (b.is_w()) cut = true;
+        }
+    }
+  return cut;
+}
+
+WaveGeom wave_geometry(const LaunchSpec& S, int g) {
+  WaveGeom W;
+  const Group &A = S.groups[g], &B = S.groups[g + 1];
+  const Task& last = S.tasks[B.end - 1];
+  const Arg& sa = space_arg(last);
+  W.nd = sa.nd;
+  int64_t elems = 1;
+  for (int d = 0; d < W.nd; ++d) {
+    W.ext[d] = std::min(last.dom[d] * sa.part.tile[d] + sa.part.off[d], sa.part.vhi[d]) - origin_of(sa, d);
+    if (W.ext[d] <= 0) return W;
+    elems *= W.ext[d];
+  }
+  if (elems < kWaveMinElems || elems >= (int64_t(1) << 31)) return W;
+  const int cd = W.nd - 1;
+  // vector width: every row of every store in memory starts on a vector
+  size_t esz = 0;
+  bool aligned = true;
+  for (int i = A.begin; i < B.end; ++i)
+    for (const Arg& a : S.tasks[i].args) {
+      if (a.imm || a.nd == 0) continue;
+      const size_t es = dtype_size(a.dtype);
+      if (esz && es != esz) return W;
+      esz = es;
+    }
+  const int vec = (int)(16 / esz);
+  for (int i = A.begin; i < B.end; ++i)
+    for (const Arg& a : S.tasks[i].args) {
+      if (a.imm || a.nd == 0) continue;
+      const LaunchRoot& r = S.roots[S.root_index.at(a.root)];
+      if (r.temp) continue;
+      if (!r.aligned16) aligned = false;
+      for (int d = 0; d < cd; ++d)
+        if (r.stride[d] % vec) aligned = false;
+    }
+  W.V = aligned ? vec : 1;
+  int phase = -1;
+  for (int i = A.begin; i < B.end; ++i) {
+    const Arg& a = S.tasks[i].args.back();
+    if (S.roots[S.root_index.at(a.root)].temp) continue;
+    const int ph = (int)(origin_of(a, cd) % W.V);
+    if (phase >= 0 && ph != phase) return W;  // written views in different vector frames
+    phase = ph;
+  }
+  W.lead = std::max(phase, 0);
+  // slices per cell: a tile costs its CTA one round of flags whatever its
+  // size, so more points per thread are better until registers spill or too
+  // few warps stay (251^3 FP32, us per sweep at 256 threads: R = 2 67, 4 42,
+  // 8 46; FP64 238, 242, 257).  1024-thread CTAs have 64 registers a thread.
+  W.R = S.block >= 1024 ? 2 : 4;
+  W.lines = W.nd == 3 ? W.ext[1] : 1;
+  W.nvx = (W.lead + W.ext[cd] + W.V - 1) / W.V;
+  const int64_t nrb = (W.ext[0] + W.R - 1) / W.R, BD = S.block - 32;  // cells per tile
+  W.cells = nrb * W.lines * W.nvx;
+  W.tiles = (W.cells + BD - 1) / BD;
+  if (W.tiles > kWaveTilesMax || W.cells >= (int64_t(1) << 31) - BD) return W;
+  // which tiles read tile t: a cell reads at every offset (read view's origin
+  // less the written view's), as a range of cell numbers, hence of tiles
+  std::set<int64_t> rel;
+  for (int i = A.begin; i < A.end; ++i)
+    for (const Arg& a : S.tasks[i].args) {
+      if (a.imm || a.nd == 0 || !a.is_r()) continue;
+      for (int j = B.begin; j < B.end; ++j) {
+        const Arg& b = S.tasks[j].args.back();
+        if (b.root != a.root || b.part == a.part) continue;
+        const int64_t d0 = origin_of(a, 0) - origin_of(b, 0), dc = origin_of(a, cd) - origin_of(b, cd);
+        const int64_t d1 = W.nd == 3 ? origin_of(a, 1) - origin_of(b, 1) : 0;
+        const int64_t v0 = floor_div(dc, W.V), v1 = floor_div(W.V - 1 + dc, W.V);
+        for (int64_t b0 = floor_div(d0, W.R); b0 <= floor_div(W.R - 1 + d0, W.R); ++b0) {
+          const int64_t o = (b0 * W.lines + d1) * W.nvx;
+          for (int64_t k = floor_div(-(o + v1), BD); k <= floor_div(BD - 1 - (o + v0), BD); ++k)
+            if (k != 0) rel.insert(k);
+          if (rel.size() > 4096) return W;
+        }
+      }
+    }
+  for (int64_t k : rel) {
+    W.reach = std::max(W.reach, k < 0 ? -k : k);
+    if (!W.readers.empty() && W.readers.back().second + 1 == k) W.readers.back().second = k;
+    else W.readers.push_back({k, k});
+  }
+  // progress: a CTA waits for the readers of its previous tile before it
+  // publishes its next one, `grid` tiles on, so a tile's readers must lie
+  // less than a grid ahead (or every tile has a CTA of its own)
+  W.min_blocks = S.min_blocks > 0 ? S.min_blocks : std::max(1, 1024 / S.block);
+  const int64_t resident = (int64_t)W.min_blocks * S.sms;
+  W.ok = W.tiles <= resident || W.reach < resident;
+  return W;
+}
+
+MarchGeom march_geometry(const LaunchSpec& S, int g) {
+  MarchGeom M;
+  const Group &A = S.groups[g], &B = S.groups[g + 1];
+  const Arg& out = S.tasks[B.end - 1].args.back();
+  if (out.nd != 2) return M;
+  const LaunchRoot& X = S.roots[S.root_index.at(out.root)];
+  if (X.temp) return M;
+  M.w0 = origin_of(out, 0);
+  M.wc = origin_of(out, 1);
+  const Task& last = S.tasks[B.end - 1];
+  M.rows = std::min(last.dom[0] * out.part.tile[0] + out.part.off[0], out.part.vhi[0]) - M.w0;
+  M.cols = std::min(last.dom[1] * out.part.tile[1] + out.part.off[1], out.part.vhi[1]) - M.wc;
+  if (M.rows <= 0 || M.cols <= 0 || M.rows * M.cols < kWaveMinElems) return M;
+  const size_t esz = dtype_size(out.dtype);
+  const int vec = (int)(16 / esz);
+  M.V = X.aligned16 && X.stride[0] % vec == 0 ? vec : 1;
+  const int64_t lead = M.wc % M.V, nv = M.V > 1 ? X.stride[0] / M.V : X.shape[1];
+  std::set<std::pair<int64_t, int64_t>> edges;
+  for (int i = A.begin; i < B.end; ++i)
+    for (size_t ai = 0; ai < S.tasks[i].args.size(); ++ai) {
+      const Arg& a = S.tasks[i].args[ai];
+      if (a.imm || a.nd == 0) continue;
+      if (S.roots[S.root_index.at(a.root)].temp) continue;
+      if (a.root != out.root || a.dtype != out.dtype) return M;
+      if (ai + 1 == S.tasks[i].args.size()) {
+        if (!(a.part == out.part)) return M;
+        continue;
+      }
+      const int64_t d0 = origin_of(a, 0) - M.w0, dc = origin_of(a, 1) - M.wc;
+      if (d0 < -1 || d0 > 1 || dc < -M.V || dc > M.V) return M;
+      if (dc < 0) M.edge_m = true;
+      if (dc > 0) M.edge_p = true;
+      for (int l = 0; l < M.V; ++l)
+        if (floor_div(dc + l, M.V)) edges.insert({floor_div(dc + l, M.V), (dc + l + M.V) % M.V});
+    }
+  // vectors of a row: the written ones and the neighbours they read, as far
+  // as the row has them
+  const int64_t f0 = (M.wc - lead) / M.V, f1 = f0 + (lead + M.cols + M.V - 1) / M.V;
+  M.pv0 = std::max<int64_t>(0, f0 - (M.edge_m ? 1 : 0));
+  M.NC = std::min(nv, f1 + (M.edge_p ? 1 : 0)) - M.pv0;
+  // threads, vectors per thread and rows ahead, from the registers of one CTA
+  // per SM; narrow rows leave room for several bands in a CTA, and rows wider
+  // than a CTA's registers are split into panels
+  const int64_t words = M.V * (int64_t)esz / 4, 
+                avail = std::min<int64_t>(255, 65536 / (S.block * std::max(1, S.min_blocks))) - 44;
+  const int64_t kmax = avail / (words * 5);  // three rows around the computed one and two ahead
+  if (kmax < 1) return M;
+  const int64_t want = (M.NC + S.block - 1) / S.block;
+  M.PN = (want + kmax - 1) / kmax;
+  const int64_t per = (M.NC + M.PN - 1) / M.PN;
+  M.K = (int)((per + S.block - 1) / S.block);
+  M.GT = (int)(((per + M.K - 1) / M.K + 31) / 32 * 32);
+  M.PC = (int64_t)M.K * M.GT;
+  M.PN = (M.NC + M.PC - 1) / M.PC;
+  M.G = M.PN > 1 ? 1 : S.block / M.GT;
+  const int64_t per_sm = S.min_blocks > 0 ? S.min_blocks : 1;
+  const int64_t ctas = std::max<int64_t>(1, per_sm * S.sms / M.PN);
+  if (M.PN > per_sm * S.sms) return M;
+  M.BR = (M.rows + ctas * M.G - 1) / (ctas * M.G);
+  M.NB = ((M.rows + M.BR - 1) / M.BR + M.G - 1) / M.G;
+  M.D = (int)std::min<int64_t>({6, avail / (words * M.K) - 3, M.BR});
+  // static shared memory: the row below the band, the warps' edge elements
+  // and, between panels, the neighbours' edge columns
+  const int64_t smem = (int64_t)M.K * S.block * M.V * esz + (3 + M.D) * (int64_t)edges.size() * M.K * (S.block / 32) * esz +
+                       (M.PN > 1 ? (M.BR + 2) * (int64_t)edges.size() * esz : 0);
+  M.smem = smem;
+  if (smem > 40 * 1024 || M.NB * M.PN > kWaveTilesMax) return M;
+  M.ok = true;
+  return M;
+}
+
+namespace {
+
+// The band form of `sweeps` in-place sweeps in a row (MarchGeom): groups g,
+// g+1 and the alike pairs after them, as one loop.  Between two of them the
+// neighbours' "stored" flags take the place of a grid barrier.
+void Gen::emit_march(int g, int sweeps) {
+  const MarchGeom M = march_geometry(S, g);
+  const Group &A = S.groups[g], &B = S.groups[g + 1];
+  const int BD = S.block, V = M.V, K = M.K, RS = 3 + M.D, NW = BD / 32;
+  const int steps = (int)std::min<int64_t>(RS, M.BR);  // rows per trip of the unrolled row loop
+  Nest n;
+  n.first = A.begin;
+  n.last = B.end;
+  n.dims = 2;
+  n.vec = V;
+  n.rank = 2;
+  BodyEnv E;
+  std::set<std::string> written, seen;
+  std::string okey;
+  const Arg* out = &S.tasks[B.end - 1].args.back();
+  for (int i = n.first; i < n.last; ++i) {
+    const Task& t = S.tasks[i];
+    for (size_t ai = 0; ai < t.args.size(); ++ai) {
+      const Arg& a = t.args[ai];
+      if (a.imm || a.nd == 0) continue;
+      const std::string k = akey(a);
+      if (ai + 1 == t.args.size()) {
+        written.insert(k);
+        if (!R(a.root).temp) okey = k;
+      } else if (!written.count(k) && seen.insert(k).second) {
+        E.reads.push_back({k, &a, "m" + std::to_string(E.reads.size()), false});
+      }
+    }
+  }
+  const LaunchRoot& X = R(out->root);
+  const int dt = out->dtype;
+  const std::string T1 = T(dt), TV = V == 4 ? "f32x4" : (V == 2 ? "f64x2" : T1);
+  const std::string ldv = V == 4 ? "ld4" : (V == 2 ? "ld2" : "ld"), stv = V == 4 ? "st4" : "st2";
+  const std::string ind = "      ", in2 = "        ", in3 = "            ";
+  // elements of neighbouring vectors: (row offset, before/after, element)
+  std::map<std::pair<int, int>, int> eidx;  // (dv, e) -> edge slot
+  std::set<std::tuple<int, int, int>> need;
+  auto src = [&](const Rd& rd, int l) {
+    const int64_t d0 = origin_of(*rd.a, 0) - M.w0, q = origin_of(*rd.a, 1) - M.wc + l;
+    const int dv = (int)floor_div(q, V);
+    return std::make_tuple((int)d0, dv, (int)(q - (int64_t)dv * V));
+  };
+  for (const Rd& rd : E.reads)
+    for (int l = 0; l < V; ++l) {
+      const auto s = src(rd, l);
+      if (std::get<1>(s) == 0) continue;
+      eidx.emplace(std::make_pair(std::get<1>(s), std::get<2>(s)), (int)eidx.size());
+      need.insert(s);
+    }
+  const int NE = (int)eidx.size();
+  const int st0 = kc.nwaves + 1;  // "edges read"; the next value: "stored"
+  kc.nwaves += 2 * sweeps;
+  kc.wave_tiles = std::max(kc.wave_tiles, M.NB * M.PN);
+  kc.march_ctas = std::max(kc.march_ctas, M.NB * M.PN);
+  wave_blocks = std::max(wave_blocks, 1);
+  const std::string sfx = std::to_string(g);
+  o << "    { // groups " << g << ", " << g + 1 << ": tasks " << n.first << ".." << n.last - 1 << ", one in-place sweep of "
+    << M.NB * M.G << " bands of " << M.BR << " rows, " << M.PN << " panel(s), " << K << " vector(s) per thread, " << M.D
+    << " row(s) ahead\n";
+  // immediates: those of every sweep in a row
+  const int imm0 = kc.nimm, ntask = n.last - n.first;
+  for (int w = 0; w < sweeps; ++w)
+    for (int i = n.first; i < n.last; ++i)
+      for (size_t ai = 0; ai < S.tasks[i].args.size(); ++ai)
+        if (S.tasks[i].args[ai].imm) imm_expr(i + w * ntask, (int)ai, dt);
+  const int nimm = (kc.nimm - imm0) / sweeps;
+  const bool pan = M.PN > 1 && NE;
+  o << ind << T1 << "* const mb" << sfx << " = (" << T1 << "*)march_raw;  // the row below the band\n";
+  if (NE) o << ind << T1 << "* const me" << sfx << " = mb" << sfx << " + " << K * BD * V << ";  // edge elements of the warps' vectors\n";
+  if (pan) o << ind << T1 << "* const mp" << sfx << " = me" << sfx << " + " << RS * NE * K * NW << ";  // edge columns of the next panels\n";
+  o << ind << "bool mok = true;\n";
+  const std::string sw = sweeps > 1 ? "sw" : "0";
+  if (sweeps > 1) o << ind << "for (int sw = 0; sw < " << sweeps << " && mok; ++sw) {\n";
+  o << ind << "const u64 fw = ep_ + " << st0 << "ull" << (sweeps > 1 ? " + 2 * sw" : "") << ";\n";
+  for (int i = n.first, k = 0; i < n.last; ++i)
+    for (size_t ai = 0; ai < S.tasks[i].args.size(); ++ai) {
+      if (!S.tasks[i].args[ai].imm) continue;
+      const std::string nm = "k" + std::to_string(i) + "_" + std::to_string(ai);
+      o << ind << "const " << T1 << " " << nm << " = ((" << T1 << ")P.imm[" << imm0 + k++;
+      if (sweeps > 1) o << " + sw * " << nimm;
+      o << "]);\n";
+      E.immv[{i, (int)ai}] = nm;
+    }
+  o << ind << "if (blockIdx.x < " << M.NB * M.PN << "u) {\n";
+  if (sweeps > 1)
+    o << in2 << "mok = sw == 0 || march_wait(P.flags, " << M.NB << "LL, " << M.PN << "LL, fw - 1, ctl, P.timeout_ns);\n"
+      << in2 << "if (mok) {\n";
+  else
+    o << in2 << "{\n";
+  if (M.G > 1) o << in2 << "const int grp = threadIdx.x / " << M.GT << ", q = threadIdx.x - grp * " << M.GT << ";\n";
+  else o << in2 << "const int grp = 0, q = threadIdx.x;\n";
+  // threads past the last group own nothing
+  o << in2 << "const int ra = grp < " << M.G << " && q < " << M.GT << " ? min((int)((blockIdx.x / " << M.PN << "u) * " << M.G
+    << "u + grp) * " << M.BR << ", " << M.rows << ") : " << M.rows << ", rz = min(ra + " << M.BR << ", " << M.rows << ");\n";
+  o << in2 << "const bool act = ra < rz;\n";
+  o << in2 << "const int pb = (int)(blockIdx.x % " << M.PN << "u) * " << M.PC << ";\n";
+  o << in2 << "const int lane = threadIdx.x & 31, lw = q >> 5;\n";
+  // one warp's vectors k are consecutive; vectors past the row repeat its last
+  for (int k = 0; k < K; ++k) {
+    o << in2 << "const int c" << k << " = pb + " << k * M.GT << " + q;\n";
+    o << in2 << T1 << "* const x" << k << " = " << ptr(out->root) << " + (i64)" << M.w0 << " * " << X.stride[0] << "LL + (i64)(min(c" << k
+      << ", " << M.NC - 1 << ") + " << M.pv0 << ") * " << V << ";\n";
+    o << in2 << "const bool s" << k << "_ = act && c" << k << " < " << (M.PN > 1 ? "min(pb + " + std::to_string(M.PC) + ", " + std::to_string(M.NC) + ")" : std::to_string(M.NC)) << ";\n";
+    o << in2 << "const int j" << k << " = (c" << k << " + " << M.pv0 << ") * " << V << " - " << M.wc << ";\n";
+  }
+  auto sl = [&](int j, int k) { return "s" + std::to_string(((j % RS) + RS) % RS) + "_" + std::to_string(k); };
+  for (int j = 0; j < RS; ++j)
+    for (int k = 0; k < K; ++k) o << in2 << TV << " s" << j << "_" << k << (V > 1 ? " = {};\n" : " = 0;\n");
+  auto row_at = [&](int k, const std::string& r) {
+    return "x" + std::to_string(k) + " + (i64)(" + r + ") * " + std::to_string(X.stride[0]) + "LL";
+  };
+  // the rows next to the band, then the band's first rows
+  o << in2 << "if (act) {\n";
+  for (int k = 0; k < K; ++k) o << in3 << sl(0, k) << " = " << ldv << "(" << row_at(k, "max(ra - 1, " + std::to_string(-M.w0) + ")") << ");\n";
+  for (int k = 0; k < K; ++k) o << in3 << "const " << TV << " b" << k << " = " << ldv << "(" << row_at(k, "min(rz, " + std::to_string(X.shape[0] - 1 - M.w0) + ")") << ");\n";
+  for (int j = 1; j <= 1 + M.D; ++j) {
+    o << in3 << "if (ra + " << j - 1 << " < rz) {\n";
+    for (int k = 0; k < K; ++k) o << in3 << "  " << sl(j, k) << " = " << ldv << "(" << row_at(k, "ra + " + std::to_string(j - 1)) << ");\n";
+    o << in3 << "}\n";
+  }
+  auto below = [&](int k) { return "mb" + sfx + " + (" + std::to_string(k * BD) + " + threadIdx.x) * " + std::to_string(V); };
+  for (int k = 0; k < K; ++k) {
+    if (V > 1) o << in3 << stv << "(" << below(k) << ", b" << k << ");\n";
+    else o << in3 << "*(" << below(k) << ") = b" << k << ";\n";
+  }
+  for (int j = 2; j <= 1 + M.D; ++j) {
+    o << in3 << "if (ra + " << j - 1 << " == rz) {\n";
+    for (int k = 0; k < K; ++k) o << in3 << "  " << sl(j, k) << " = b" << k << ";\n";
+    o << in3 << "}\n";
+  }
+  o << in2 << "}\n";
+  if (pan) {
+    // columns: element e of the vector before (after) the panel, rows -1 .. BR
+    for (const auto& kv : eidx) {
+      const int dv = kv.first.first, e = kv.first.second;
+      const std::string v = dv < 0 ? "pb - 1" : "pb + " + std::to_string(M.PC);
+      o << in2 << "if (" << v << " >= 0 && " << v << " < " << M.NC << ")\n";
+      o << in2 << "  for (int i = threadIdx.x; i < rz - ra + 2; i += " << BD << ") mp" << sfx << "[" << kv.second * (M.BR + 2)
+        << " + i] = ld(" << ptr(out->root) << " + (i64)min(max(ra - 1 + i + " << M.w0 << ", 0), " << X.shape[0] - 1 << ") * " << X.stride[0] << "LL + (i64)(" << v << " + "
+        << M.pv0 << ") * " << V << " + " << e << ");\n";
+    }
+  }
+  auto put_edges = [&](int j, const std::string& pad) {
+    const int slot = ((j % RS) + RS) % RS;
+    for (const auto& kv : eidx) {
+      const int dv = kv.first.first, e = kv.first.second;
+      o << pad << "if (lane == " << (dv < 0 ? 31 : 0) << " && act) {";
+      for (int k = 0; k < K; ++k)
+        o << " me" << sfx << "[" << (slot * NE + kv.second) * K * NW << " + (threadIdx.x >> 5) * " << K << " + " << k << "] = " << sl(j, k)
+          << (V > 1 ? ".v[" + std::to_string(e) + "]" : std::string()) << ";";
+      o << " }\n";
+    }
+  };
+  if (NE) {
+    put_edges(0, in2);
+    put_edges(1, in2);
+  }
+  // the rows and columns next to the band have been read (and used) here
+  o << in2 << "{ u32 used_ = 0u";
+  for (int k = 0; k < K; ++k)
+    for (int l = 0; l < V; ++l) o << " ^ bits_of(" << sl(0, k) << (V > 1 ? ".v[" + std::to_string(l) + "]" : std::string()) << ")";
+  o << ";\n" << in2 << "  if (used_ == 0x7fc5a3d1u) wave_pause(); }\n";
+  o << in2 << "march_raise(P.flags, fw);\n";
+  o << in2 << "for (int n0 = 0; n0 < " << M.BR << "; n0 += " << steps << ") {\n";
+  for (int u = 0; u < steps; ++u) {
+    o << in2 << "  { // row ra + n0 + " << u << "\n";
+    o << in3 << "if (n0 + " << u << " >= " << M.BR << ") break;\n";
+    o << in3 << "const int i = ra + n0 + " << u << ";\n";
+    o << in3 << "const bool row = act && i < rz;\n";
+    // the row D + 1 below, or the saved one under the band
+    o << in3 << "if (act && i + " << M.D + 1 << " < rz) {\n";
+    for (int k = 0; k < K; ++k)
+      o << in3 << "  " << sl(u + RS - 1, k) << " = " << ldv << "(" << row_at(k, "i + " + std::to_string(M.D + 1)) << ");\n";
+    o << in3 << "} else if (act && i + " << M.D + 1 << " == rz) {\n";
+    for (int k = 0; k < K; ++k) o << in3 << "  " << sl(u + RS - 1, k) << " = " << ldv << "(" << below(k) << ");\n";
+    o << in3 << "}\n";
+    if (NE) {
+      put_edges(u + 2, in3);
+      o << in3 << "__syncthreads();\n";
+    }
+    std::map<std::tuple<int, int, int>, std::string> xv;
+    for (const auto& s : need) {
+      const int d0 = std::get<0>(s), dv = std::get<1>(s), e = std::get<2>(s), ei = eidx.at({dv, e});
+      const int slot = (u + 1 + d0 + RS) % RS;
+      const std::string nm = "x" + std::to_string(d0 + 1) + (dv < 0 ? "m" : "p") + std::to_string(e);
+      xv[s] = nm;
+      for (int k = 0; k < K; ++k) {
+        o << in3 << T1 << " " << nm << "_" << k << " = " << (dv > 0 ? "__shfl_down_sync" : "__shfl_up_sync") << "(0xffffffffu, "
+          << sl(u + 1 + d0, k) << (V > 1 ? ".v[" + std::to_string(e) + "]" : std::string()) << ", 1);\n";
+        // across warps: the neighbouring vector is in the warp before
+        // (after), or, past the group's last warp, in the next k
+        const int base = (slot * NE + ei) * K * NW;
+        const int wg = M.GT / 32;
+        const std::string w = "(int)(threadIdx.x >> 5)";
+        o << in3 << "if (lane == " << (dv > 0 ? 31 : 0) << " && act) {\n";
+        const std::string at = "me" + sfx + "[" + std::to_string(base) + " + ";
+        std::string panel = pan ? "mp" + sfx + "[" + std::to_string(ei * (M.BR + 2)) + " + i - ra + " + std::to_string(1 + d0) + "]" : "";
+        if (dv > 0) {
+          o << in3 << "  if (lw < " << wg - 1 << ") " << nm << "_" << k << " = " << at << "(" << w << " + 1) * " << K << " + " << k << "];\n";
+          if (k + 1 < K)
+            o << in3 << "  else " << nm << "_" << k << " = " << at << "(" << w << " - " << wg - 1 << ") * " << K << " + " << k + 1 << "];\n";
+          else if (pan)
+            o << in3 << "  else if (row) " << nm << "_" << k << " = " << panel << ";\n";
+        } else {
+          o << in3 << "  if (lw > 0) " << nm << "_" << k << " = " << at << "(" << w << " - 1) * " << K << " + " << k << "];\n";
+          if (k > 0)
+            o << in3 << "  else " << nm << "_" << k << " = " << at << "(" << w << " + " << wg - 1 << ") * " << K << " + " << k - 1 << "];\n";
+          else if (pan)
+            o << in3 << "  else if (row) " << nm << "_" << k << " = " << panel << ";\n";
+        }
+        o << in3 << "}\n";
+      }
+    }
+    std::vector<std::string> slots, none;
+    for (int k = 0; k < K; ++k) {
+      slots.push_back("u" + std::to_string(k));
+      none.push_back("");
+      for (const Rd& rd : E.reads) {
+        o << in3 << "const " << TV << " " << rd.var << "_u" << k << " = " << (V > 1 ? "{{" : "");
+        for (int l = 0; l < V; ++l) {
+          const auto s = src(rd, l);
+          o << (l ? ", " : "");
+          if (std::get<1>(s)) o << xv.at(s) << "_" << k;
+          else o << sl(u + 1 + std::get<0>(s), k) << (V > 1 ? ".v[" + std::to_string(std::get<2>(s)) + "]" : std::string());
+        }
+        o << (V > 1 ? "}};\n" : ";\n");
+      }
+    }
+    const auto outvars = emit_compute(n, E, V, slots, none, in3);
+    const auto& vv = outvars.at(okey);
+    if (u == 0)
+      o << in3 << "if (n0 == 0 && !(mok = march_wait(P.flags, " << M.NB << "LL, " << M.PN << "LL, fw, ctl, P.timeout_ns))) break;\n";
+    o << in3 << "if (row) {\n";
+    for (int k = 0; k < K; ++k) {
+      const std::string at = row_at(k, "i"), jn = "j" + std::to_string(k);
+      if (V == 1) {
+        o << in3 << "  if (s" << k << "_ && " << jn << " >= 0 && " << jn << " < " << M.cols << ") *(" << at << ") = " << vv[k] << ";\n";
+        continue;
+      }
+      o << in3 << "  if (s" << k << "_ && " << jn << " >= 0 && " << jn << " + " << V << " <= " << M.cols << ") " << stv << "(" << at << ", " << TV << "{{";
+      for (int l = 0; l < V; ++l) o << (l ? ", " : "") << vv[k * V + l];
+      o << "}});\n" << in3 << "  else if (s" << k << "_) {\n";
+      for (int l = 0; l < V; ++l)
+        o << in3 << "    if (" << jn << " + " << l << " >= 0 && " << jn << " + " << l << " < " << M.cols << ") *(" << at << " + " << l << ") = "
+          << vv[k * V + l] << ";\n";
+      o << in3 << "  }\n";
+    }
+    o << in3 << "}\n";
+    o << in2 << "  }\n";
+  }
+  o << in2 << "}\n";
+  if (sweeps > 1) o << in2 << "if (mok && sw + 1 < " << sweeps << ") march_raise(P.flags, fw + 1);\n";
+  o << in2 << "}\n" << ind << "}\n";
+  if (sweeps > 1) o << ind << "}\n";
+  o << ind << "if (!mok) break;\n";
+  o << "    }\n";
+}
+
+// The tasks of a sweep with its temporaries renamed: two sweeps with equal
+// signatures differ in their temporaries and immediates only.
+std::string Gen::sweep_signature(int g) const {
+  std::map<int64_t, int> temps;
+  std::string k;
+  for (int i = S.groups[g].begin; i < S.groups[g + 1].end; ++i) {
+    k += "|" + std::to_string(S.tasks[i].op);
+    for (const Arg& a : S.tasks[i].args) {
+      if (a.imm) k += ",i";
+      else if (a.nd > 0 && R(a.root).temp)
+        k += ",t" + std::to_string(temps.emplace(a.root, (int)temps.size()).first->second) + "@" + a.part.key();
+      else k += "," + akey(a);
+      k += ":" + std::to_string(a.priv);
+    }
+  }
+  return k;
+}
+
+void Gen::emit_wave(int g) {
+  const WaveGeom W = wave_geometry(S, g);
+  const Group &A = S.groups[g], &B = S.groups[g + 1];
+  const int BD = S.block - 32, V = W.V, Rr = W.R, cd = W.nd - 1;
+  Nest n;
+  n.first = A.begin;
+  n.last = B.end;
+  n.dims = 2;
+  n.vec = V;
+  n.rank = W.nd;
+  BodyEnv E;
+  std::set<std::string> written;
+  struct Out { std::string key; const Arg* a; };
+  std::vector<Out> outs;
+  std::set<std::string> seen;
+  for (int i = n.first; i < n.last; ++i) {
+    const Task& t = S.tasks[i];
+    for (size_t ai = 0; ai < t.args.size(); ++ai) {
+      const Arg& a = t.args[ai];
+      if (a.imm || a.nd == 0) continue;
+      const std::string k = akey(a);
+      const bool out = ai + 1 == t.args.size();
+      if (!out && a.is_r() && !written.count(k) && seen.insert(k).second)
+        E.reads.push_back({k, &a, "m" + std::to_string(E.reads.size()), !R(a.root).written});
+      if (out) {
+        if (written.insert(k).second && !R(a.root).temp) outs.push_back({k, &a});
+      }
+    }
+  }
+  const std::string ind = "      ", in2 = ind + "    ";
+  const int dt = outs[0].a->dtype;
+  const std::string T1 = T(dt), TV = V == 4 ? "f32x4" : (V == 2 ? "f64x2" : T1);
+  const std::string ldv = V == 4 ? "ld4" : "ld2", stv = V == 4 ? "st4" : "st2";
+  ++kc.nwaves;
+  kc.wave_tiles = std::max(kc.wave_tiles, W.tiles);
+  if (W.reach > 0) kc.wave_reach = std::max(kc.wave_reach, W.reach);
+  wave_blocks = std::max(wave_blocks, W.min_blocks);
+  o << "    { // groups " << g << ", " << g + 1 << ": tasks " << n.first << ".." << n.last - 1
+    << ", one in-place sweep of " << W.tiles << " tiles\n";
+  for (int i = n.first; i < n.last; ++i) {
+    const Task& t = S.tasks[i];
+    for (size_t ai = 0; ai < t.args.size(); ++ai) {
+      if (!t.args[ai].imm) continue;
+      const std::string nm = "k" + std::to_string(i) + "_" + std::to_string(ai);
+      o << ind << "const " << T1 << " " << nm << " = " << imm_expr(i, (int)ai, dt) << ";\n";
+      E.immv[{i, (int)ai}] = nm;
+    }
+  }
+  o << ind << "const u64 fw = ep_ + " << kc.nwaves << "ull;\n";
+  // the ordering warp
+  int64_t nflag = 0;
+  for (const auto& rr : W.readers) nflag += rr.second - rr.first + 1;
+  o << ind << "if (threadIdx.x >= " << BD << ") {\n";
+  o << ind << "  for (i64 t = blockIdx.x; t < " << W.tiles << "LL; t += gridDim.x, ++wrd_) {\n";
+  o << ind << "    bool ok_ = wave_raise(&wsync_, wrd_, P.flags + t, ctl, fw, P.timeout_ns);\n";
+  if (nflag > 0) {
+    o << ind << "    for (int i = threadIdx.x & 31; i < " << nflag << " && ok_; i += 32) {\n";
+    o << ind << "      const i64 u = t + i + (";
+    int64_t at = 0;
+    for (size_t k = 0; k < W.readers.size(); ++k) {
+      const std::string v = std::to_string(W.readers[k].first - at) + "LL";
+      at += W.readers[k].second - W.readers[k].first + 1;
+      o << (k + 1 < W.readers.size() ? "i < " + std::to_string(at) + " ? " + v + " : " : v);
+    }
+    o << ");\n";
+    o << ind << "      if (u >= 0 && u < " << W.tiles << "LL && !wave_poll(P.flags + u, fw, ctl, P.timeout_ns)) ok_ = false;\n";
+    o << ind << "    }\n";
+  }
+  o << ind << "    if (!wave_release(&wsync_, wrd_, ok_, ctl, fw)) break;\n";
+  o << ind << "  }\n";
+  o << ind << "} else {\n";
+  o << ind << "bool live = false;\n" << ind << "u32 prb = 0, py = 0, pjv = 0;\n";
+  o << ind << "bool pact = false;\n";
+  for (size_t k = 0; k < outs.size(); ++k)
+    for (int u = 0; u < Rr; ++u) o << ind << TV << " h" << k << "_" << u << (V > 1 ? " = {};\n" : " = 0;\n");
+  o << ind << "for (i64 t = blockIdx.x;; t += gridDim.x) {\n";
+  o << ind << "  const bool have = t < " << W.tiles << "LL;\n";
+  // threads past the last cell repeat it (their results are not stored)
+  o << ind << "  const u32 c = have ? min((u32)t * " << BD << "u + threadIdx.x, " << W.cells - 1 << "u) : 0u;\n";
+  o << ind << "  const u32 rb = c / " << W.lines * W.nvx << "u;\n";
+  if (W.nd == 3) {
+    o << ind << "  const u32 rem = c - rb * " << W.lines * W.nvx << "u;\n";
+    o << ind << "  const u32 y = rem / " << W.nvx << "u;\n" << ind << "  const u32 jv = rem - y * " << W.nvx << "u;\n";
+  } else {
+    o << ind << "  const u32 y = 0, jv = c - rb * " << W.nvx << "u;\n";
+  }
+  for (size_t k = 0; k < outs.size(); ++k)
+    for (int u = 0; u < Rr; ++u) o << ind << "  " << TV << " n" << k << "_" << u << (V > 1 ? " = {};\n" : " = 0;\n");
+  o << ind << "  if (have) {\n";
+  // loads: distinct (root, slice, line, vector), one element where only one
+  // of the vector is used
+  struct Ld { std::string var; bool scalar = false; int elem = 0; bool ro = false; std::set<int> need; int64_t root; int64_t k0, o1, vb; };
+  std::map<std::string, int> lidx;
+  std::vector<Ld> loads;
+  auto want = [&](const Rd& rd, int64_t k0, int64_t o1, int64_t vb, int e) -> int {
+    const std::string k = std::to_string(rd.a->root) + "," + std::to_string(k0) + "," + std::to_string(o1) + "," + std::to_string(vb);
+    auto it = lidx.find(k);
+    if (it == lidx.end()) {
+      Ld L;
+      L.var = "w" + std::to_string(loads.size());
+      L.ro = rd.ro;
+      L.root = rd.a->root;
+      L.k0 = k0;
+      L.o1 = o1;
+      L.vb = vb;
+      it = lidx.emplace(k, (int)loads.size()).first;
+      loads.push_back(L);
+    }
+    loads[it->second].need.insert(e);
+    return it->second;
+  };
+  // element of lane l of read rd in slot u: (load, element)
+  auto source = [&](const Rd& rd, int u, int l) {
+    const int64_t q = origin_of(*rd.a, cd) - W.lead + l;
+    const int64_t vb = floor_div(q, V);
+    const int e = (int)(q - vb * V);
+    return std::make_pair(want(rd, origin_of(*rd.a, 0) + u, W.nd == 3 ? origin_of(*rd.a, 1) : 0, vb, e), e);
+  };
+  for (int u = 0; u < Rr; ++u)
+    for (const Rd& rd : E.reads)
+      for (int l = 0; l < V; ++l) source(rd, u, l);
+  std::map<std::string, std::string> rowp, colv;
+  int nrow = 0;
+  for (Ld& L : loads) {
+    const LaunchRoot& r = R(L.root);
+    const std::string rk = std::to_string(L.root) + "," + std::to_string(L.k0) + "," + std::to_string(L.o1);
+    if (!rowp.count(rk)) {
+      const std::string nm = "p" + std::to_string(nrow++);
+      o << in2 << "const " << T1 << "* " << nm << " = " << ptr(L.root) << " + ";
+      const std::string row = "rb * " + std::to_string(Rr) + "u + " + std::to_string(L.k0) + "u";
+      // slices past the end (a ragged last block) repeat the store's last one
+      if (W.ext[0] % Rr) o << "(i64)min(" << row << ", " << r.shape[0] - 1 << "u)";
+      else o << "(i64)(" << row << ")";
+      o << " * " << r.stride[0] << "LL";
+      if (W.nd == 3) o << " + (i64)(y + " << L.o1 << "u) * " << r.stride[1] << "LL";
+      o << ";\n";
+      rowp[rk] = nm;
+    }
+    // vectors before the row's first or after its last serve no valid lane:
+    // clamped into the row
+    const int64_t nv = V > 1 ? r.stride[cd - 1] / V : r.shape[cd];
+    const bool lo = L.vb < 0, hi = W.nvx - 1 + L.vb > nv - 1;
+    const std::string ck = std::to_string(L.vb) + (lo ? "l" : "") + (hi ? "h" + std::to_string(nv) : "");
+    if (!colv.count(ck)) {
+      const std::string nm = "c" + std::to_string(colv.size());
+      std::string e = "((int)jv + " + std::to_string(L.vb) + ")";
+      if (lo) e = "max(" + e + ", 0)";
+      if (hi) e = "min(" + e + ", " + std::to_string(nv - 1) + ")";
+      o << in2 << "const int " << nm << " = " << e << " * " << V << ";\n";
+      colv[ck] = nm;
+    }
+    const std::string ad = rowp[rk] + " + " + colv[ck];
+    L.scalar = V > 1 && L.need.size() == 1;
+    if (L.scalar) {
+      L.elem = *L.need.begin();
+      o << in2 << "const " << T1 << " " << L.var << " = " << (L.ro ? "ldro(" : "ld(") << ad << " + " << L.elem << ");\n";
+    } else if (V > 1) {
+      o << in2 << "const " << TV << " " << L.var << " = " << ldv << (L.ro ? "ro(" : "(") << ad << ");\n";
+    } else {
+      o << in2 << "const " << T1 << " " << L.var << " = " << (L.ro ? "ldro(" : "ld(") << ad << ");\n";
+    }
+  }
+  // assemble the lanes, compute, keep the results
+  std::vector<std::string> slots, none;
+  for (int u = 0; u < Rr; ++u) {
+    slots.push_back("u" + std::to_string(u));
+    none.push_back("");
+    for (const Rd& rd : E.reads) {
+      o << in2 << "const " << TV << " " << rd.var << "_u" << u << " = ";
+      if (V > 1) o << "{{";
+      for (int l = 0; l < V; ++l) {
+        const auto se = source(rd, u, l);
+        const Ld& L = loads[se.first];
+        o << (l ? ", " : "") << L.var;
+        if (V > 1 && !L.scalar) o << ".v[" << se.second << "]";
+      }
+      o << (V > 1 ? "}};\n" : ";\n");
+    }
+  }
+  const auto outvars = emit_compute(n, E, V, slots, none, in2);
+  for (size_t k = 0; k < outs.size(); ++k) {
+    const auto& vv = outvars.at(outs[k].key);
+    for (int u = 0; u < Rr; ++u) {
+      const std::string h = "n" + std::to_string(k) + "_" + std::to_string(u);
+      if (V == 1) o << in2 << h << " = " << vv[u] << ";\n";
+      else
+        for (int l = 0; l < V; ++l) o << in2 << h << ".v[" << l << "] = " << vv[u * V + l] << ";\n";
+    }
+  }
+  o << ind << "  wave_read_done(&wsync_, wrd_ + (live ? 1u : 0u), 0u";
+  for (size_t k = 0; k < outs.size(); ++k)
+    for (int u = 0; u < Rr; ++u)
+      for (int l = 0; l < V; ++l)
+        o << " ^ bits_of(n" << k << "_" << u << (V > 1 ? ".v[" + std::to_string(l) + "]" : std::string()) << ")";
+  o << ");\n";
+  o << ind << "  }\n";
+  // the previous tile's results, once every tile that reads it has read
+  o << ind << "  if (live) {\n";
+  o << ind << "    if (!wave_ready(&wsync_, wrd_, ctl, fw, P.timeout_ns)) break;\n";
+  o << ind << "    ++wrd_;\n";
+  o << ind << "    if (pact) {\n";
+  for (size_t k = 0; k < outs.size(); ++k) {
+    const Arg& a = *outs[k].a;
+    const LaunchRoot& r = R(a.root);
+    o << ind << "      {\n";
+    o << ind << "        " << T1 << "* q_ = " << ptr(a.root) << " + (i64)(prb * " << Rr << "u + " << origin_of(a, 0) << "u) * "
+      << r.stride[0] << "LL";
+    if (W.nd == 3) o << " + (i64)(py + " << origin_of(a, 1) << "u) * " << r.stride[1] << "LL";
+    o << " + (i64)pjv * " << V << " + " << origin_of(a, cd) - W.lead << ";\n";
+    o << ind << "        const int j_ = (int)pjv * " << V << " - " << W.lead << ";\n";
+    for (int u = 0; u < Rr; ++u) {
+      const std::string h = "h" + std::to_string(k) + "_" + std::to_string(u);
+      const std::string at_ = "q_ + " + std::to_string(u * r.stride[0]) + "LL";
+      o << ind << "        ";
+      if (W.ext[0] % Rr) o << "if (prb * " << Rr << "u + " << u << "u < " << W.ext[0] << "u) ";
+      if (V == 1) {
+        o << "*(" << at_ << ") = " << h << ";\n";
+        continue;
+      }
+      o << "{\n";
+      o << ind << "          if (j_ >= 0 && j_ + " << V << " <= " << W.ext[cd] << ") " << stv << "(" << at_ << ", " << h << ");\n";
+      o << ind << "          else {\n";
+      for (int l = 0; l < V; ++l)
+        o << ind << "            if (j_ + " << l << " >= 0 && j_ + " << l << " < " << W.ext[cd] << ") *(" << at_ << " + " << l
+          << ") = " << h << ".v[" << l << "];\n";
+      o << ind << "          }\n" << ind << "        }\n";
+    }
+    o << ind << "      }\n";
+  }
+  o << ind << "    }\n" << ind << "  }\n";
+  o << ind << "  if (!have) break;\n";
+  for (size_t k = 0; k < outs.size(); ++k)
+    for (int u = 0; u < Rr; ++u) o << ind << "  h" << k << "_" << u << " = n" << k << "_" << u << ";\n";
+  o << ind << "  live = true;\n";
+  o << ind << "  pact = (u32)t * " << BD << "u + threadIdx.x < " << W.cells << "u;\n";
+  o << ind << "  prb = rb;\n" << ind << "  py = y;\n" << ind << "  pjv = jv;\n";
+  o << ind << "}\n";
+  o << ind << "}\n" << ind << "__syncthreads();\n";
+  o << ind << "if (wsync_.fail) break;\n";
+  o << "    }\n";
+}
+
 KernelCode Gen::run() {
   emit_params();
   std::ostringstream body;
@@ -1083,6 +1847,19 @@ KernelCode Gen::run() {
     o << "  xstage_init(&xs_mbar_);\n";
   }
   emit_prologue();
+  for (const Group& G : S.groups)
+    if (G.wave) {
+      o << "  const u64 ep_ = ctl->epoch;  // the last CTA to exit moves it on\n";
+      o << "  __shared__ __align__(8) WaveSync wsync_;\n  u32 wrd_ = 0;\n  wave_init(&wsync_);\n";
+      break;
+    }
+  int64_t march_smem = 0;
+  for (int g = 0; g + 1 < (int)S.groups.size(); ++g)
+    if (S.groups[g].wave) {
+      const MarchGeom M = march_geometry(S, g);
+      if (M.ok) march_smem = std::max(march_smem, M.smem);
+    }
+  if (march_smem) o << "  __shared__ __align__(16) unsigned char march_raw[" << march_smem << "];\n";
   o << "  do {\n";
   for (int g = 0; g < (int)S.groups.size(); ++g) {
     if (g > 0 && !S.groups[g - 1].scalar) {
@@ -1094,6 +1871,22 @@ KernelCode Gen::run() {
         g = h - 1;
         continue;
       }
+    }
+    if (S.groups[g].wave) {
+      if (march_geometry(S, g).ok) {
+        int sweeps = 1;
+        const std::string sig = sweep_signature(g);
+        while (g + 2 * sweeps + 1 < (int)S.groups.size() && S.groups[g + 2 * sweeps].wave &&
+               S.groups[g + 2 * sweeps + 1].end - S.groups[g + 2 * sweeps].begin == S.groups[g + 1].end - S.groups[g].begin &&
+               sweep_signature(g + 2 * sweeps) == sig)
+          ++sweeps;
+        emit_march(g, sweeps);
+        g += 2 * sweeps - 1;
+        continue;
+      }
+      emit_wave(g);
+      ++g;
+      continue;
     }
     emit_group(g);
   }
@@ -1109,6 +1902,7 @@ KernelCode Gen::run() {
     if (!r.zero_d || !r.live_out || r.param < 0) continue;
     o << "      *" << ptr(r.root) << " = " << sreg.at(r.root) << ";\n";
   }
+  if (kc.nwaves) o << "      ctl->epoch = ep_ + " << kc.nwaves << "ull;\n";
   o << "    }\n";
   o << "    ctl_reset(ctl);\n";
   o << "  }\n";
@@ -1117,13 +1911,15 @@ KernelCode Gen::run() {
   std::ostringstream src;
   src << "#include \"dfs_device.cuh\"\nusing namespace dfs;\n";
   src << "struct Params {\n  void* p[" << std::max(1, kc.nptr) << "];\n  double imm[" << std::max(1, kc.nimm)
-      << "];\n  void* partials;\n  Ctl* ctl;\n  u64 timeout_ns;\n  i64 red_stride;\n};\n";
+      << "];\n  void* partials;\n  Ctl* ctl;\n  u64 timeout_ns;\n  i64 red_stride;\n"
+      << (kc.nwaves ? "  u64* flags;\n" : "") << "};\n";
   const std::string body_s = o.str();
   const size_t h = std::hash<std::string>{}(body_s);
   char nm[64];
   snprintf(nm, sizeof nm, "dfs_k%016zx", h);
   kc.name = nm;
-  src << "extern \"C\" __global__ void __launch_bounds__(" << S.block << (S.min_blocks > 0 ? ", " + std::to_string(S.min_blocks) : std::string()) << ") " << kc.name
+  const int min_blocks = S.min_blocks > 0 ? S.min_blocks : wave_blocks;
+  src << "extern \"C\" __global__ void __launch_bounds__(" << S.block << (min_blocks > 0 ? ", " + std::to_string(min_blocks) : std::string()) << ") " << kc.name
       << "(const __grid_constant__ Params P) {\n"
       << body_s << "}\n";
   kc.source = src.str();

@@ -402,7 +402,8 @@ struct Ctl {
   u32 exit_arrive;  // CTAs that finished the launch
   int err;          // first device error (0 = none)
   int err_where;    // barrier index that timed out
-  u64 pad[2];
+  u64 epoch;        // in-place sweeps run so far (values of their flags; kept across launches)
+  u64 pad;
   u64 ticket[kTickets];  // work-queue counters, one per dynamically dealt phase
 };
 
@@ -422,7 +423,7 @@ __device__ __forceinline__ int ld_relaxed_int(const int* p) {
   return v;
 }
 
-enum { ERR_BARRIER_TIMEOUT = 1 };
+enum { ERR_BARRIER_TIMEOUT = 1, ERR_WAVE_TIMEOUT = 3 };
 
 __device__ __forceinline__ void red_release_add_u32(u32* p, u32 v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
@@ -467,6 +468,150 @@ __device__ __forceinline__ bool grid_barrier(Ctl* ctl, u32 k, u64 timeout_ns, bo
   }
   __syncthreads();
   return s_ok != 0;
+}
+
+// ------------------------------------------------------------- mbarriers
+__device__ __forceinline__ u32 smem_u32(const void* p) { return (u32)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(u64* mbar, u32 count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(u64* mbar) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(u64* mbar, u32 phase) {
+  u32 done;
+  asm volatile(
+      "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+      : "=r"(done)
+      : "r"(smem_u32(mbar)), "r"(phase)
+      : "memory");
+  return done != 0;
+}
+
+// Waits for a phase, at most timeout_ns.
+__device__ __forceinline__ bool mbar_wait(u64* mbar, u32 phase, u64 timeout_ns) {
+  if (mbar_try(mbar, phase)) return true;
+  const u64 t0 = globaltimer_ns();
+  while (!mbar_try(mbar, phase))
+    if (globaltimer_ns() - t0 > timeout_ns) return false;
+  return true;
+}
+
+// ------------------------------------------------------- in-place sweeps
+// A CTA of a sweep (codegen.cpp, WaveGeom) is `block - 32` threads that load,
+// compute and store cells, and one warp that keeps the tiles in order.  Per
+// tile (round): every working warp arrives on `read` once its loads have
+// returned; the ordering warp waits for that, raises the tile's flag, waits
+// for the flags of the tiles that read this one, and arrives on `ready`; the
+// working warps wait for it only after they have read the next tile, and then
+// store.  So the flag's fence and the polling (a microsecond or more under
+// load) pass while the next tile is being read.
+struct WaveSync {
+  u64 read[2], ready[2];  // mbarriers of even and odd rounds: a warp may be a round ahead of another
+  int fail;
+};
+
+// Every load of the tile precedes its warp's arrival on `read`, which the
+// caller has waited for, so the release orders them before the flag, and the
+// acquire in wave_poll before any store that overwrites what they read.
+// Flags hold the number of the last sweep that set them (64 bits, never
+// reset), so no launch has to clear them.
+__device__ __forceinline__ void wave_publish(u64* flag, u64 want) {
+  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(flag), "l"(want) : "memory");
+}
+__device__ __forceinline__ u64 ld_acquire_u64(const u64* p) {
+  u64 v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+// Waits for a flag, at most timeout_ns (or until any CTA records an error).
+__device__ __forceinline__ bool wave_poll(const u64* flag, u64 want, Ctl* ctl, u64 timeout_ns) {
+  if (ld_acquire_u64(flag) == want) return true;
+  const u64 t0 = globaltimer_ns();
+  while (ld_acquire_u64(flag) != want) {
+    if (ld_relaxed_int(&ctl->err) != 0) return false;
+    if (globaltimer_ns() - t0 > timeout_ns) return false;
+  }
+  return true;
+}
+__device__ __forceinline__ void wave_error(WaveSync* w, Ctl* ctl, u64 want) {
+  if (atomicCAS(&ctl->err, 0, (int)ERR_WAVE_TIMEOUT) == 0) ctl->err_where = (int)(want & 0x7fffffff);
+  *(volatile int*)&w->fail = 1;
+}
+// Once per kernel, by every thread, before the first sweep.
+__device__ __forceinline__ void wave_init(WaveSync* w) {
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&w->read[i], blockDim.x / 32 - 1);
+      mbar_init(&w->ready[i], 1);
+    }
+    w->fail = 0;
+  }
+  __syncthreads();
+}
+// A working warp before it stores its part of a tile: true when it may.  The
+// limit is the ordering warp's own (the arrival on `read`, then the flags),
+// which arrives on `ready` even when it gives up.
+__device__ __forceinline__ bool wave_ready(WaveSync* w, u32 round, Ctl* ctl, u64 want, u64 timeout_ns) {
+  if (!mbar_wait(&w->ready[round & 1], (round >> 1) & 1, 3 * timeout_ns)) wave_error(w, ctl, want);
+  return *(volatile int*)&w->fail == 0;
+}
+__device__ __forceinline__ void wave_pause() { asm volatile("nanosleep.u32 0;" ::: "memory"); }
+// A working warp whose loads of a tile have returned: `used` combines every
+// value computed from them, and the branch on it keeps the arrival behind the
+// loads' completion, not only behind their issue.
+__device__ __forceinline__ u32 bits_of(float v) { return (u32)__float_as_int(v); }
+__device__ __forceinline__ u32 bits_of(double v) {
+  const u64 b = (u64)__double_as_longlong(v);
+  return (u32)b ^ (u32)(b >> 32);
+}
+__device__ __forceinline__ void wave_read_done(WaveSync* w, u32 round, u32 used) {
+  if (used == 0x7fc5a3d1u) wave_pause();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(&w->read[round & 1]);
+}
+// The ordering warp, for one tile: waits until its CTA has read it and raises
+// its flag ...
+__device__ __forceinline__ bool wave_raise(WaveSync* w, u32 round, u64* flag, Ctl* ctl, u64 want, u64 timeout_ns) {
+  const bool ok = mbar_wait(&w->read[round & 1], (round >> 1) & 1, timeout_ns);
+  if (!ok) wave_error(w, ctl, want);
+  else if ((threadIdx.x & 31) == 0) wave_publish(flag, want);
+  return ok;
+}
+// ... and, after polling the readers' flags, lets the tile be stored.
+__device__ __forceinline__ bool wave_release(WaveSync* w, u32 round, bool ok, Ctl* ctl, u64 want) {
+  ok = __all_sync(0xffffffffu, ok);
+  if ((threadIdx.x & 31) == 0) {
+    if (!ok) wave_error(w, ctl, want);
+    mbar_arrive(&w->ready[round & 1]);
+  }
+  return ok;
+}
+
+// Bands (codegen.cpp, MarchGeom).  Waits until the up to eight neighbours of
+// band b, panel p have reached stage `want` (flags only grow).  Called by
+// every thread; the acquire orders the neighbours' stores (stage "stored")
+// before the loads that follow, and their loads (stage "read") before the
+// stores that follow.
+__device__ __forceinline__ bool march_wait(const u64* flags, i64 nb, i64 np, u64 want, Ctl* ctl, u64 timeout_ns) {
+  bool ok = true;
+  if (threadIdx.x < 9) {
+    const i64 b = (i64)blockIdx.x / np + (i64)(threadIdx.x / 3) - 1, p = (i64)blockIdx.x % np + (i64)(threadIdx.x % 3) - 1;
+    if (b >= 0 && b < nb && p >= 0 && p < np && threadIdx.x != 4) {
+      const u64* f = flags + b * np + p;
+      const u64 t0 = globaltimer_ns();
+      while (ok && ld_acquire_u64(f) < want)
+        if (ld_relaxed_int(&ctl->err) != 0 || globaltimer_ns() - t0 > timeout_ns) ok = false;
+      if (!ok && atomicCAS(&ctl->err, 0, (int)ERR_WAVE_TIMEOUT) == 0) ctl->err_where = (int)(want & 0x7fffffff);
+    }
+  }
+  return __syncthreads_and(ok ? 1 : 0) != 0;
+}
+// This CTA has reached a stage.
+__device__ __forceinline__ void march_raise(u64* flags, u64 stage) {
+  __syncthreads();
+  if (threadIdx.x == 0) wave_publish(flags + blockIdx.x, stage);
 }
 
 // Kernel exit: returns true in exactly one CTA -- the last to arrive -- after
@@ -520,8 +665,6 @@ struct XWin {
 
 enum { ERR_COPY_TIMEOUT = 2 };
 
-__device__ __forceinline__ u32 smem_u32(const void* p) { return (u32)__cvta_generic_to_shared(p); }
-
 // Once per CTA, by every thread, before the first xstage.
 __device__ __forceinline__ void xstage_init(u64* mbar) {
   if (threadIdx.x == 0) {
@@ -530,16 +673,6 @@ __device__ __forceinline__ void xstage_init(u64* mbar) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
-}
-
-__device__ __forceinline__ bool mbar_try(u64* mbar, u32 phase) {
-  u32 done;
-  asm volatile(
-      "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-      : "=r"(done)
-      : "r"(smem_u32(mbar)), "r"(phase)
-      : "memory");
-  return done != 0;
 }
 
 // Stages the point's windows (record w: lo0, len0, lo1, len1, lo2, len2 in

@@ -30,6 +30,7 @@ struct CachedLaunch {
   int block = 256;
   int grid = 1;
   bool cooperative = false;
+  bool waves = false;  // takes the context's flag array
   int nbarriers = 0;
   int nptr = 0, nimm = 0;
   std::vector<int> ptr_canon;                 // canonical root id per pointer param
@@ -79,6 +80,7 @@ struct dfs_ctx {
   dfs::Ctl* ctl = nullptr;
   void* partials = nullptr;
   size_t partials_cap = 0;
+  uint64_t* flags = nullptr;  // one per tile of an in-place sweep (kWaveTilesMax), zeroed once
   std::unordered_map<std::string, std::unique_ptr<dfs::CachedWindow>> wcache;
   dfs::Stats st;
   std::string last_source;
@@ -431,7 +433,7 @@ std::string plan_json(const Plan& p, const std::vector<Task>& w, const WindowInf
 // role of every root (pointer parameter, temporary, 0-d value loaded before
 // or published after the launch).  `valid` is the value state before it.
 LaunchSpec make_spec(dfs_ctx* c, const std::vector<Task>& w, const std::map<int64_t, RootInfo>& roots,
-                     const Plan& P, int g0, int g1, std::map<int64_t, bool>& valid) {
+                     const Plan& P, int g0, int g1, std::map<int64_t, bool>& valid, bool waves = false) {
   const int t0 = P.groups[g0].begin, t1 = P.groups[g1 - 1].end;
   LaunchSpec spec;
   spec.block = c->cfg.block_threads;
@@ -439,6 +441,7 @@ LaunchSpec make_spec(dfs_ctx* c, const std::vector<Task>& w, const std::map<int6
   spec.unroll = c->cfg.unroll;
   spec.persistent = (g1 - g0) > 1;
   spec.debug_skip = c->cfg.debug_skip_arrival;
+  spec.sms = c->sms;
   for (int i = t0; i < t1; ++i) spec.tasks.push_back(w[i]);
   for (int g = g0; g < g1; ++g) {
     Group G = P.groups[g];
@@ -457,7 +460,6 @@ LaunchSpec make_spec(dfs_ctx* c, const std::vector<Task>& w, const std::map<int6
       if (P.temps.count({g, r})) tcount[r].second++;
     }
   }
-  int nparam = 0;
   for (int i = t0; i < t1; ++i)
     for (const Arg& a : w[i].args) {
       if (a.imm || spec.root_index.count(a.root)) continue;
@@ -477,43 +479,78 @@ LaunchSpec make_spec(dfs_ctx* c, const std::vector<Task>& w, const std::map<int6
       spec.root_index[a.root] = (int)spec.roots.size();
       spec.roots.push_back(lr);
     }
-  for (LaunchRoot& lr : spec.roots) {
-    for (int i = t0; i < t1; ++i)
-      for (const Arg& a : w[i].args) {
-        if (a.imm || a.root != lr.root) continue;
-        lr.written |= a.is_w() || a.is_rd();
-        lr.read |= a.is_r();
+  // in-place sweeps: pairs of groups cut by an anti-dependence (WaveGeom)
+  if (waves && c->cfg.fusion)
+    for (int k = 0; k + 1 < (int)spec.groups.size(); ++k)
+      if (wave_legal(spec, k)) {
+        spec.groups[k].wave = true;
+        ++k;
       }
-    const auto& tc = tcount[lr.root];
-    const RootInfo& ri = roots.at(lr.root);
-    if (lr.zero_d) {
-      // 0-d values live in registers; memory is needed to load a prior value
-      // or to publish the result beyond this launch
-      bool used_later = false;
-      for (int i = t1; i < (int)w.size(); ++i)
-        for (const Arg& a : w[i].args)
-          if (!a.imm && a.root == lr.root && (a.is_r() || a.is_rd())) used_later = true;
-      lr.live_out = lr.written && (ri.app_live || ri.wrapped || used_later);
-      lr.temp = !lr.live_out;
-      bool load = false;
-      if (lr.valid_before) {
-        // first access in program order decides whether the old value is used
-        for (int i = t0; i < t1 && !load; ++i) {
-          bool touched = false;
-          for (const Arg& a : w[i].args) {
-            if (a.imm || a.root != lr.root) continue;
-            touched = true;
-            if (a.is_r() || a.is_rd()) load = true;
-          }
-          if (touched) break;
-        }
-      }
-      lr.valid_before = lr.valid_before && load;
-      if (load || lr.live_out) lr.param = nparam++;
-    } else {
-      lr.temp = c->cfg.fusion && tc.first > 0 && tc.first == tc.second;
-      if (!lr.temp) lr.param = nparam++;
+  // a store that only the two groups of a sweep use, and that Def. 4 makes a
+  // temporary of the two together
+  auto pair_temp = [&](int64_t root) {
+    for (int k = 0; k + 1 < (int)spec.groups.size(); ++k) {
+      if (!spec.groups[k].wave) continue;
+      const int b = spec.groups[k].begin, e = spec.groups[k + 1].end;
+      bool inside = false, outside = false;
+      for (int i = 0; i < (int)spec.tasks.size(); ++i)
+        for (const Arg& a : spec.tasks[i].args)
+          if (!a.imm && a.root == root) (i >= b && i < e ? inside : outside) = true;
+      if (inside) return !outside && is_temporary(w, t0 + b, t0 + e, root, roots.at(root));
     }
+    return false;
+  };
+  const std::map<int64_t, bool> valid0 = valid;
+  for (bool again = true; again;) {
+    again = false;
+    int nparam = 0;
+    for (LaunchRoot& lr : spec.roots) {
+      lr.param = -1;
+      lr.valid_before = valid0.at(lr.root);
+    }
+    for (LaunchRoot& lr : spec.roots) {
+      for (int i = t0; i < t1; ++i)
+        for (const Arg& a : w[i].args) {
+          if (a.imm || a.root != lr.root) continue;
+          lr.written |= a.is_w() || a.is_rd();
+          lr.read |= a.is_r();
+        }
+      const auto& tc = tcount[lr.root];
+      const RootInfo& ri = roots.at(lr.root);
+      if (lr.zero_d) {
+        // 0-d values live in registers; memory is needed to load a prior value
+        // or to publish the result beyond this launch
+        bool used_later = false;
+        for (int i = t1; i < (int)w.size(); ++i)
+          for (const Arg& a : w[i].args)
+            if (!a.imm && a.root == lr.root && (a.is_r() || a.is_rd())) used_later = true;
+        lr.live_out = lr.written && (ri.app_live || ri.wrapped || used_later);
+        lr.temp = !lr.live_out;
+        bool load = false;
+        if (lr.valid_before) {
+          // first access in program order decides whether the old value is used
+          for (int i = t0; i < t1 && !load; ++i) {
+            bool touched = false;
+            for (const Arg& a : w[i].args) {
+              if (a.imm || a.root != lr.root) continue;
+              touched = true;
+              if (a.is_r() || a.is_rd()) load = true;
+            }
+            if (touched) break;
+          }
+        }
+        lr.valid_before = lr.valid_before && load;
+        if (load || lr.live_out) lr.param = nparam++;
+      } else {
+        lr.temp = c->cfg.fusion && tc.first > 0 && (tc.first == tc.second || pair_temp(lr.root));
+        if (!lr.temp) lr.param = nparam++;
+      }
+    }
+    for (int k = 0; k < (int)spec.groups.size(); ++k)
+      if (spec.groups[k].wave && !march_geometry(spec, k).ok && !wave_geometry(spec, k).ok) {
+        spec.groups[k].wave = false;
+        again = true;  // the pair's temporaries go back to memory
+      }
   }
   return spec;
 }
@@ -530,7 +567,7 @@ int build_window(dfs_ctx* c, const WindowInfo& wi, std::unique_ptr<CachedWindow>
   for (size_t li = 0; li < P.launches.size(); ++li) {
     const int g0 = P.launches[li].first, g1 = P.launches[li].second;
     const int t0 = P.groups[g0].begin, t1 = P.groups[g1 - 1].end;
-    LaunchSpec spec = make_spec(c, w, wi.roots, P, g0, g1, valid);
+    LaunchSpec spec = make_spec(c, w, wi.roots, P, g0, g1, valid, true);
     for (const LaunchRoot& lr : spec.roots)
       if (lr.param >= 0) need_mem.insert(lr.root);
     KernelCode kc;
@@ -553,18 +590,22 @@ int build_window(dfs_ctx* c, const WindowInfo& wi, std::unique_ptr<CachedWindow>
     L.name = kc.name;
     L.block = spec.block;
     L.nbarriers = kc.nbarriers;
-    L.cooperative = kc.nbarriers > 0;
+    L.waves = kc.nwaves > 0;
+    L.cooperative = kc.nbarriers > 0 || L.waves;
     bool all_scalar = true;
     for (const Group& G : spec.groups) all_scalar &= G.scalar;
     // per-point groups want one CTA per point (more CTAs would only wait at
     // the barriers); kernels made only of flat sweeps use every resident CTA
     int64_t want = 1;
     if (!all_scalar) want = kc.has_points ? kc.max_points : (kc.has_flat ? INT64_MAX : 1);
+    want = std::max(want, kc.wave_tiles);
     int per_sm = comp->occupancy > 0 ? comp->occupancy : 1;
     if (c->cfg.ctas_per_sm > 0) per_sm = std::min(per_sm, c->cfg.ctas_per_sm);
     const int64_t cap = (int64_t)per_sm * c->sms;
     if (L.cooperative && comp->occupancy <= 0) return fail(c, DFS_ERR_CUDA, "generated kernel cannot be resident for a cooperative launch");
     L.grid = (int)std::max<int64_t>(1, std::min(want, cap));
+    if (L.waves && (kc.march_ctas > L.grid || (kc.wave_tiles > L.grid && kc.wave_reach >= L.grid)))
+      return fail(c, DFS_ERR_CUDA, "too few resident CTAs for an in-place sweep");
     L.nptr = kc.nptr;
     L.nimm = kc.nimm;
     for (int64_t r : kc.ptr_roots) L.ptr_canon.push_back(wi.canon.at(r));
@@ -587,6 +628,19 @@ int build_window(dfs_ctx* c, const WindowInfo& wi, std::unique_ptr<CachedWindow>
   return DFS_OK;
 }
 
+// The flag array of in-place sweeps: fixed size, so graphs that recorded its
+// address stay valid; allocated with the first sweep, or before a capture.
+int reserve_flags(dfs_ctx* c) {
+  if (c->flags) return DFS_OK;
+  if (c->capturing) return fail(c, DFS_ERR_STATE, "sweep flags missing inside a capture");
+  void* p = nullptr;
+  const size_t n = (size_t)kWaveTilesMax * sizeof(uint64_t);
+  CUDA_OK(cudaMallocAsync(&p, n, c->stream));
+  c->flags = (uint64_t*)p;
+  CUDA_OK(cudaMemsetAsync(p, 0, n, c->stream));
+  return DFS_OK;
+}
+
 int run_window(dfs_ctx* c, const CachedWindow& cw, const WindowInfo& wi) {
   c->lastb.ok = false;
   for (int id : cw.materialise) {
@@ -604,7 +658,11 @@ int run_window(dfs_ctx* c, const CachedWindow& cw, const WindowInfo& wi) {
       CUDA_OK(cudaMallocAsync(&c->partials, cap, c->stream));
       c->partials_cap = cap;
     }
-    std::vector<uint64_t> blob((size_t)std::max(1, L.nptr) + (size_t)std::max(1, L.nimm) + 4, 0);
+    if (L.waves) {
+      const int rc = reserve_flags(c);
+      if (rc) return rc;
+    }
+    std::vector<uint64_t> blob((size_t)std::max(1, L.nptr) + (size_t)std::max(1, L.nimm) + 5, 0);
     for (int i = 0; i < L.nptr; ++i) {
       const StoreRec& r = c->stores.at(wi.by_canon[L.ptr_canon[i]]);
       void* p = r.ptr;
@@ -624,6 +682,7 @@ int run_window(dfs_ctx* c, const CachedWindow& cw, const WindowInfo& wi) {
     blob[tb + 2] = to;
     const int64_t rs = L.red_stride;
     std::memcpy(&blob[tb + 3], &rs, sizeof rs);
+    std::memcpy(&blob[tb + 4], &c->flags, sizeof c->flags);
     void* bp = blob.data();
     void* params[] = {bp};
     // the kernel takes one struct parameter: pass its bytes as the argument
@@ -1059,6 +1118,7 @@ int flush_batch(dfs_ctx* c) {
       return fail(c, DFS_ERR_STATE, "batch scratch would grow inside a capture: run the batch once before");
     }
     if (sval_need > c->sval_cap) {
+      if (c->flags) cudaFreeAsync(c->flags, c->stream);
       if (c->sval) cudaFreeAsync(c->sval, c->stream);
       CUDA_OK(cudaMallocAsync((void**)&c->sval, sval_need, c->stream));
       c->sval_cap = sval_need;
@@ -1653,8 +1713,11 @@ static int check_device_error(dfs_ctx* c) {
   Ctl h;
   CUDA_OK(cudaMemcpy(&h, c->ctl, sizeof h, cudaMemcpyDeviceToHost));
   if (h.err != 0) {
-    cudaMemset(c->ctl, 0, sizeof(Ctl));
+    cudaMemset(c->ctl, 0, sizeof(Ctl));  // sweep numbers start again, so the flags do too
+    if (c->flags) cudaMemset(c->flags, 0, (size_t)kWaveTilesMax * sizeof(uint64_t));
     cudaDeviceSynchronize();
+    if (h.err == 3)
+      return fail(c, DFS_ERR_BARRIER_TIMEOUT, "an in-place sweep timed out waiting for a neighbouring tile");
     if (h.err == 2)
       return fail(c, DFS_ERR_BARRIER_TIMEOUT, "a staged SpMV copy of x did not complete in time");
     return fail(c, DFS_ERR_BARRIER_TIMEOUT, "a grid barrier timed out (barrier " + std::to_string(h.err_where) + ")");
@@ -1900,6 +1963,8 @@ int dfs_capture_begin(dfs_ctx* c) {
       CUDA_OK(cudaMallocAsync(&c->partials, want, c->stream));
       c->partials_cap = want;
     }
+    rc = reserve_flags(c);
+    if (rc) return rc;
     CUDA_OK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     c->capturing = true;
     c->captured_allocs.clear();

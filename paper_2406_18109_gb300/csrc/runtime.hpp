@@ -102,7 +102,8 @@ struct Ctl {
   uint32_t exit_arrive;
   int32_t err;
   int32_t err_where;
-  uint64_t pad[2];
+  uint64_t epoch;
+  uint64_t pad;
   uint64_t ticket[16];
 };
 
@@ -110,6 +111,7 @@ struct Ctl {
 struct Group {  // one fused task (a fusible prefix, Section 4.2.2)
   int begin = 0, end = 0;
   bool scalar = false;
+  bool wave = false;  // launch packing: runs with the next group as one in-place sweep (WaveGeom)
 };
 
 struct Plan {
@@ -172,7 +174,56 @@ struct LaunchSpec {
   bool persistent = false;
   int debug_skip = 0;  // test hook: CTA 0 withholds its arrival at this barrier
   int min_blocks = 0;  // > 0: __launch_bounds__ minimum resident CTAs per SM (caps registers)
+  int sms = 152;       // SMs of the device (co-resident CTAs of an in-place sweep)
 };
+
+// Two consecutive vector groups A, B that the anti-dependence constraint cut
+// (B writes the store whose shifted views A reads, as in Fig. 1) run as ONE
+// in-place sweep ("wave") instead of two phases with a grid barrier between
+// them.  The iteration space is cut into cells of R slices of dimension 0 by
+// one vector of the last dimension, numbered row-major; a tile is `block`
+// consecutive cells, one per thread, and tile t belongs to CTA t mod grid.  A
+// CTA computes a tile's results in registers, publishes a flag ("tile t has
+// read its neighbourhood"), and stores the results one round later, once the
+// flags of every tile that reads tile t are up.  The results never pass
+// through memory between the groups, and the store A hands to B is a
+// temporary of the pair (Def. 4 over both).
+struct WaveGeom {
+  bool ok = false;
+  int nd = 0, V = 1, R = 1, lead = 0;      // lead: columns before the written views in their first vector
+  int64_t ext[MAXD] = {1, 1, 1};
+  int64_t lines = 1, nvx = 0, cells = 0, tiles = 0;
+  std::vector<std::pair<int64_t, int64_t>> readers;  // ranges of u - t over the tiles u that read tile t
+  int64_t reach = 0;                       // largest |u - t|
+  int min_blocks = 1;                      // CTAs per SM the kernel is compiled to keep resident
+};
+// Legality (dependences of the tasks, one shared iteration space) of running
+// groups g and g+1 of the launch as a wave.
+bool wave_legal(const LaunchSpec& spec, int g);
+// Its cells and tiles, once the launch's temporaries are known; ok = false
+// when the wave cannot make progress (it reaches further than the co-resident
+// CTAs) or does not pay.
+WaveGeom wave_geometry(const LaunchSpec& spec, int g);
+
+// The 2-D form of a wave whose only store in memory is the written one: bands
+// of rows.  A thread owns K vectors of a row and keeps the rows around the one
+// it computes in registers, so every row is read once and written once, and a
+// CTA only has to agree with its neighbours on the rows (and, where a row is
+// split into panels, columns) at the edges of its band: it reads those before
+// its first store, raises a flag, and waits for its neighbours' flags.
+struct MarchGeom {
+  bool ok = false;
+  int V = 1, K = 1, D = 1, G = 1, GT = 32;  // D: rows read ahead; G groups of GT threads, a band each
+  int64_t rows = 0, cols = 0;              // written rectangle
+  int64_t BR = 1, NB = 1, PN = 1;          // rows per band, CTAs along rows, panels of a row
+  int64_t pv0 = 0, NC = 0, PC = 0;         // first root vector, vectors of a row, of a panel
+  int64_t w0 = 0, wc = 0;                  // origin of the written view in its root
+  int64_t smem = 0;
+  bool edge_m = false, edge_p = false;     // elements of the vector before / after are needed
+};
+MarchGeom march_geometry(const LaunchSpec& spec, int g);
+constexpr int64_t kWaveTilesMax = 1 << 19;  // flags of a context (8 bytes each)
+constexpr int64_t kWaveMinElems = 4096;
 
 struct KernelCode {
   std::string name;
@@ -185,6 +236,10 @@ struct KernelCode {
   bool has_flat = false;    // some group sweeps a flat range
   bool has_points = false;  // some group deals points to CTAs (max_points of them)
   int nbarriers = 0;
+  int nwaves = 0;           // flag values the in-place sweeps use (> 0: the kernel takes the flag array)
+  int64_t wave_tiles = 0;   // most tiles of one sweep
+  int64_t march_ctas = 0;   // CTAs that must be resident for the bands of a sweep
+  int64_t wave_reach = 0;   // most CTAs a sweep with more tiles than CTAs needs beyond a tile's own
   std::vector<int64_t> red_points;  // points of each reduction slot
   std::vector<double> imms;         // immediate values in parameter order
   std::vector<std::pair<int, int>> imm_src;  // (task, arg) of each immediate param
