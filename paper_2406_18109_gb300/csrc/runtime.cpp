@@ -567,24 +567,37 @@ int build_window(dfs_ctx* c, const WindowInfo& wi, std::unique_ptr<CachedWindow>
   for (size_t li = 0; li < P.launches.size(); ++li) {
     const int g0 = P.launches[li].first, g1 = P.launches[li].second;
     const int t0 = P.groups[g0].begin, t1 = P.groups[g1 - 1].end;
-    LaunchSpec spec = make_spec(c, w, wi.roots, P, g0, g1, valid, true);
+    LaunchSpec spec;
+    KernelCode kc;
+    const Compiled* comp = nullptr;
+    // In-place sweeps need their CTAs resident together; where the built
+    // kernel does not reach the residency the geometry counted on (a
+    // ctas_per_sm beyond what shared memory or threads allow), the launch is
+    // generated again with two phases per sweep.
+    for (const bool waves : {true, false}) {
+      spec = make_spec(c, w, wi.roots, P, g0, g1, valid, waves);
+      try {
+        kc = generate(spec);
+      } catch (const std::exception& e) {
+        return fail(c, DFS_ERR_INVALID, std::string("code generation: ") + e.what());
+      }
+      std::string err;
+      c->last_source = kc.source;
+      if (!c->device) {
+        // analysis-only context: check that the kernel compiles for the target
+        if (!c->jit->compile_only(kc.source, kc.name, err)) return fail(c, DFS_ERR_COMPILE, err);
+        break;
+      }
+      comp = c->jit->get(kc.source, kc.name, spec.block, err, kc.dyn_smem);
+      if (!comp) return fail(c, DFS_ERR_COMPILE, err);
+      if (kc.nwaves == 0) break;
+      const int64_t resident =
+          (int64_t)(c->cfg.ctas_per_sm > 0 ? std::min(comp->occupancy, c->cfg.ctas_per_sm) : comp->occupancy) * c->sms;
+      if (kc.march_ctas <= resident && (kc.wave_tiles <= resident || kc.wave_reach < resident)) break;
+    }
     for (const LaunchRoot& lr : spec.roots)
       if (lr.param >= 0) need_mem.insert(lr.root);
-    KernelCode kc;
-    try {
-      kc = generate(spec);
-    } catch (const std::exception& e) {
-      return fail(c, DFS_ERR_INVALID, std::string("code generation: ") + e.what());
-    }
-    std::string err;
-    c->last_source = kc.source;
-    if (!c->device) {
-      // analysis-only context: check that the kernel compiles for the target
-      if (!c->jit->compile_only(kc.source, kc.name, err)) return fail(c, DFS_ERR_COMPILE, err);
-      continue;
-    }
-    const Compiled* comp = c->jit->get(kc.source, kc.name, spec.block, err, kc.dyn_smem);
-    if (!comp) return fail(c, DFS_ERR_COMPILE, err);
+    if (!c->device) continue;
     CachedLaunch L;
     L.k = comp;
     L.name = kc.name;
@@ -604,8 +617,6 @@ int build_window(dfs_ctx* c, const WindowInfo& wi, std::unique_ptr<CachedWindow>
     const int64_t cap = (int64_t)per_sm * c->sms;
     if (L.cooperative && comp->occupancy <= 0) return fail(c, DFS_ERR_CUDA, "generated kernel cannot be resident for a cooperative launch");
     L.grid = (int)std::max<int64_t>(1, std::min(want, cap));
-    if (L.waves && (kc.march_ctas > L.grid || (kc.wave_tiles > L.grid && kc.wave_reach >= L.grid)))
-      return fail(c, DFS_ERR_CUDA, "too few resident CTAs for an in-place sweep");
     L.nptr = kc.nptr;
     L.nimm = kc.nimm;
     for (int64_t r : kc.ptr_roots) L.ptr_canon.push_back(wi.canon.at(r));
@@ -1118,7 +1129,6 @@ int flush_batch(dfs_ctx* c) {
       return fail(c, DFS_ERR_STATE, "batch scratch would grow inside a capture: run the batch once before");
     }
     if (sval_need > c->sval_cap) {
-      if (c->flags) cudaFreeAsync(c->flags, c->stream);
       if (c->sval) cudaFreeAsync(c->sval, c->stream);
       CUDA_OK(cudaMallocAsync((void**)&c->sval, sval_need, c->stream));
       c->sval_cap = sval_need;
@@ -1436,6 +1446,7 @@ int dfs_shutdown(dfs_ctx* c) {
         if (kv.second.owned && kv.second.ptr) cudaFreeAsync(kv.second.ptr, c->stream);
       if (c->partials) cudaFreeAsync(c->partials, c->stream);
       if (c->sval) cudaFreeAsync(c->sval, c->stream);
+      if (c->flags) cudaFreeAsync(c->flags, c->stream);
       for (auto& kv : c->tables) cudaFreeAsync(kv.second.dev, c->stream);
       c->tables.clear();
       cudaStreamSynchronize(c->stream);

@@ -119,3 +119,32 @@ def test_sweeps_replayed_from_a_graph(offsets, shape):
         got = g.numpy()
         rt.graph_destroy(graph)
     assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
+
+
+@pytest.mark.parametrize("shape, offsets", [((515, 700), FIVE), ((40, 70, 81), SEVEN)], ids=["2d", "3d"])
+@pytest.mark.parametrize("kw", [dict(ctas_per_sm=8), dict(ctas_per_sm=4, block=1024), dict(ctas_per_sm=16, block=128)], ids=str)
+def test_sweeps_with_more_ctas_asked_than_fit(shape, offsets, kw):
+    """A ctas_per_sm that the sweep's kernel cannot reach: two phases then."""
+    _check(shape, np.float32, offsets, kw, wave=None)
+
+
+def test_sweeps_around_a_batch_that_grows_its_scratch():
+    """A batch reallocates its own scratch only: the sweeps' flags stay."""
+    from paper_2406_18109_gb300 import arrays as A
+    host = np.random.default_rng(6).uniform(0.0, 1.0, (203, 517)).astype(np.float32)
+    want, _ = _run("unfused", host, FIVE, 6, 1, False)
+    with gpu_runtime("persistent") as rt:
+        g = rt.array(host)
+        views = _views(g, FIVE)
+        for count in (1, 3, 40):
+            for _ in range(2):
+                _sweep(views)
+                rt.flush()
+            vs = [rt.array(np.full(3000, i, dtype=np.float32)) for i in range(count)]
+            rt.batch_begin()
+            for v in vs:
+                v *= A.dot(v, v)
+                rt.batch_next()
+            rt.batch_end()
+        got = g.numpy()
+    assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
