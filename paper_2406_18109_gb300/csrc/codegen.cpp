@@ -1029,7 +1029,7 @@ void Gen::emit_finalise(const char* ind) {
   o << ind << "if (threadIdx.x < 32) {\n";
   for (size_t j = 0; j < pending_red.size(); ++j) {
     const Red& r = pending_red[j];
-    o << ind << "  const " << T(r.dtype) << " " << bc[j] << "_t = sum_partials((const " << T(r.dtype)
+    o << ind << "  const " << T(r.dtype) << " " << bc[j] << "_t = sum_partials8((const " << T(r.dtype)
       << "*)P.partials + " << r.slot << "LL * P.red_stride, " << r.points << "LL);\n";
     o << ind << "  if (threadIdx.x == 0) " << bc[j] << " = " << bc[j] << "_t;\n";
   }
@@ -1073,7 +1073,7 @@ int Gen::emit_warp0_scalars(int g) {
   o << "    if (threadIdx.x < 32) {\n";
   for (const Red& r : pending_red) {
     const std::string nm = sreg.at(r.root);
-    o << "      { const " << T(r.dtype) << " tot = sum_partials((const " << T(r.dtype) << "*)P.partials + "
+    o << "      { const " << T(r.dtype) << " tot = sum_partials8((const " << T(r.dtype) << "*)P.partials + "
       << r.slot << "LL * P.red_stride, " << r.points << "LL);\n";
     if (have[r.root])
       o << "        " << nm << " = op_add(" << nm << ", tot); }\n";

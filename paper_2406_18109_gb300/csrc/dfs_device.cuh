@@ -802,3 +802,24 @@ template <typename T> __device__ __forceinline__ T sum_partials(const T* partial
 }
 
 }  // namespace dfs
+// The same sum (the same bits) with eight loads in flight per lane: every CTA
+// of a single launch waits for it between two phases.  One 0-d result of 582
+// FP64 partials took 2.3 to 6 us of a 76 us CG iteration, so 1.3 to 3.3 (CG at
+// 256^2, 128 partials: 12.6 -> 11.0 us per iteration, with two such sums).
+// Batched kernels keep the short form: one warp per instance sums, and the
+// registers of eight loads cost BiCGSTAB windows more than they save (3.32 ->
+// 3.37 ms for eight iterations of four 3-D solves).
+template <typename T> __device__ __forceinline__ T sum_partials8(const T* partials, i64 n) {
+  const int l = threadIdx.x & 31;
+  T acc = T(0);
+  for (i64 at = l; at < n; at += 256) {
+    T v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (at + 32 * u < n) v[u] = ld(partials + at + 32 * u);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (at + 32 * u < n) acc += v[u];
+  }
+  return warp_sum_xor(acc);
+}
