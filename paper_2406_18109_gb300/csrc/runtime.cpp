@@ -940,6 +940,31 @@ int flush_batch(dfs_ctx* c) {
   if (c->cfg.launch_mode != DFS_LAUNCH_PERSISTENT || !c->cfg.fusion) return fallback("batching runs fused, persistent launches");
   const int K = (int)inst.size();
   std::vector<std::vector<Task>> iw(K);
+  // Points are dealt in the order of the instances, and a phase ends with its
+  // slowest point: those with the most entries go first, unless all have about
+  // the same.  (2048 rows of about 16 scattered entries take 100 us; dealt
+  // last, they ended an SpMV phase at 282 us whose CTAs were done at 187 on
+  // average; first, at 210.)
+  {
+    std::vector<int64_t> work(inst.size(), 0);
+    for (size_t k = 0; k < inst.size(); ++k)
+      for (size_t i = inst[k].first; i < inst[k].second; ++i) {
+        const Task& t = w[i];
+        if (t.op != DFS_OP_SPMV || t.args[4].part.kind != 1) continue;
+        const NPart &cp = t.args[1].part, &rp = t.args[0].part;
+        const int64_t nnz = cp.vhi[0] - cp.vlo[0], rows = std::max<int64_t>(1, rp.vhi[0] - rp.vlo[0] - 1);
+        work[k] = std::max(work[k], (int64_t)((double)std::min(t.args[4].part.tile[0], rows) * (double)nnz / (double)rows));
+      }
+    const auto mm = std::minmax_element(work.begin(), work.end());
+    if (*mm.second > *mm.first + *mm.first / 2) {
+      std::vector<size_t> at(inst.size());
+      for (size_t k = 0; k < at.size(); ++k) at[k] = k;
+      std::stable_sort(at.begin(), at.end(), [&](size_t a, size_t b) { return work[a] > work[b]; });
+      std::vector<std::pair<size_t, size_t>> sorted;
+      for (size_t k : at) sorted.push_back(inst[k]);
+      inst = std::move(sorted);
+    }
+  }
   std::vector<std::map<int64_t, RootInfo>> iroots(K);
   std::vector<std::vector<int64_t>> canon(K);
   for (int i = 0; i < K; ++i) {
