@@ -585,18 +585,23 @@ bool BatchGen::run(BatchCode& out, std::string& why) {
   // the last CTA finishes what remains and publishes the 0-d results
   o << "  if (last_cta(ctl)) {\n";
   o << "    if (ld_relaxed_int(&ctl->err) == 0) {\n";
-  o << "      const int lane = threadIdx.x & 31;\n";
-  o << "      for (i64 inst = threadIdx.x >> 5; inst < NI; inst += " << S.block / 32 << ") {\n";
+  // a warp per instance where sums are still to be finished, else a thread:
+  // one CTA walks all instances, and each step is a chain of dependent loads
+  const bool sums = !pending.empty();
+  if (sums) o << "      const int lane = threadIdx.x & 31;\n";
+  o << "      for (i64 inst = threadIdx.x" << (sums ? " >> 5" : "") << "; inst < NI; inst += " << (sums ? S.block / 32 : S.block)
+    << ") {\n";
   o << "        const Inst& D = P.insts[inst];\n";
   o << "        double* sv = P.sval + inst * " << std::max(1, bc.nsval) << "LL;\n";
   local.clear();
   finals("    ");
-  o << "        if (lane == 0) {\n";
+  if (sums) o << "        if (lane == 0) {\n";
   for (const LaunchRoot& r : S.roots) {
     if (!r.zero_d || !r.live_out || r.param < 0) continue;
     o << "          *(" << T(r.dtype) << "*)D.p[" << r.param << "] = " << zero_d_read(r.root, r.dtype, true) << ";\n";
   }
-  o << "        }\n      }\n    }\n    ctl_reset(ctl);\n  }\n";
+  if (sums) o << "        }\n";
+  o << "      }\n    }\n    ctl_reset(ctl);\n  }\n";
   bc.nbarriers = nbar;
   bc.vec = V;
 
