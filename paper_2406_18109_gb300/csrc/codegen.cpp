@@ -1891,10 +1891,25 @@ KernelCode Gen::run() {
     emit_group(g);
   }
   o << "  } while (0);\n";
-  o << "  if (last_cta(ctl)) {\n";
-  if (!pending_red.empty()) {
-    o << "    if (ld_relaxed_int(&ctl->err) == 0) {\n";
-    emit_finalise("      ");
+  // The exit count costs every launch a round trip to L2 after its last store;
+  // a kernel without barriers, sums, scalars to publish or sweeps leaves the
+  // control block as it found it (Black-Scholes, 1,000,003 options: 10.25 ->
+  // 9.79 us).
+  bool exits = nbar > 0 || !pending_red.empty() || kc.nwaves > 0;
+  for (const LaunchRoot& r : S.roots) exits = exits || (r.zero_d && r.live_out && r.param >= 0);
+  if (exits) {
+    o << "  if (last_cta(ctl)) {\n";
+    if (!pending_red.empty()) {
+      o << "    if (ld_relaxed_int(&ctl->err) == 0) {\n";
+      emit_finalise("      ");
+      o << "    }\n";
+    }
+    o << "    if (threadIdx.x == 0) {\n";
+    for (const LaunchRoot& r : S.roots) {
+      if (!r.zero_d || !r.live_out || r.param < 0) continue;
+      o << "      *" << ptr(r.root) << " = " << sreg.at(r.root) << ";\n";
+    }
+    if (kc.nwaves) o << "      ctl->epoch = ep_ + " << kc.nwaves << "ull;\n";
     o << "    }\n";
   }
   o << "    if (threadIdx.x == 0) {\n";
