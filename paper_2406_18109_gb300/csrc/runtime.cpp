@@ -552,6 +552,8 @@ LaunchSpec make_spec(dfs_ctx* c, const std::vector<Task>& w, const std::map<int6
         again = true;  // the pair's temporaries go back to memory
       }
   }
+  if (waves && c->cfg.fusion && std::none_of(spec.groups.begin(), spec.groups.end(), [](const Group& G) { return G.wave; }))
+    pack_groups(spec);
   return spec;
 }
 
@@ -620,7 +622,7 @@ int build_window(dfs_ctx* c, const WindowInfo& wi, std::unique_ptr<CachedWindow>
     L.nptr = kc.nptr;
     L.nimm = kc.nimm;
     for (int64_t r : kc.ptr_roots) L.ptr_canon.push_back(wi.canon.at(r));
-    for (const auto& s : kc.imm_src) L.imm_src.push_back({s.first + t0, s.second});
+    for (const auto& s : kc.imm_src) L.imm_src.push_back({(spec.order.empty() ? s.first : spec.order[s.first]) + t0, s.second});
     int64_t stride = 1;
     for (int64_t p : kc.red_points) stride = std::max(stride, p);
     L.red_stride = stride;

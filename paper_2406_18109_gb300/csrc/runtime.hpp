@@ -167,6 +167,7 @@ struct LaunchRoot {  // one root buffer used by a launch
 struct LaunchSpec {
   std::vector<Task> tasks;         // tasks of the launch in program order
   std::vector<Group> groups;       // re-based on `tasks`
+  std::vector<int> order;          // when groups were joined (pack_groups): a task's place in the window's order
   std::vector<LaunchRoot> roots;   // indexed through root_index
   std::map<int64_t, int> root_index;
   int block = 256;
@@ -224,6 +225,10 @@ struct MarchGeom {
 MarchGeom march_geometry(const LaunchSpec& spec, int g);
 constexpr int64_t kWaveTilesMax = 1 << 19;  // flags of a context (8 bytes each)
 constexpr int64_t kWaveMinElems = 4096;
+
+// Launch packing: joins groups that can share one sweep although scalar tasks
+// or other sweeps stand between them.  Results keep their bits.
+void pack_groups(LaunchSpec& spec);
 
 struct KernelCode {
   std::string name;
