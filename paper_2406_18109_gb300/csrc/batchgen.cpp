@@ -58,6 +58,7 @@ class BatchGen {
   int nbar = 0;
   int nreg = 0;
   bool stage = false;  // some SpMV carries x windows, staged in shared memory
+  bool by_rows = false;  // SpMVs are computed a warp's rows at a time (spmv_rows)
 
   const LaunchRoot& R(int64_t r) const { return S.roots[S.root_index.at(r)]; }
   std::string T(int dt) const { return dtype_cname(dt); }
@@ -422,26 +423,38 @@ void BatchGen::vector_group(int g) {
       }
     };
     bool has_spmv = false;
-    for (int k = i; k < j; ++k) has_spmv = has_spmv || (coop && S.tasks[k].op == DFS_OP_SPMV);
+    for (int k = i; k < j; ++k) has_spmv = has_spmv || ((coop || by_rows) && S.tasks[k].op == DFS_OP_SPMV);
     if (has_spmv) {
       // SpMV rows shared by lanes (spmv_warp, lanes per row from the
-      // instance's descriptor).  Elements are dealt to threads as in the
+      // instance's descriptor), or a warp's rows summed from shared memory
+      // (spmv_rows).  Elements are dealt to threads as in the
       // plain loops (vectors of V, then the scalar tail), so fused reductions
       // sum in the same order; a warp takes 32 consecutive vectors per trip
       o << ind << "  const int lane_ = threadIdx.x & 31;\n";
-      auto coop_spmv = [&](int w, const std::string& first, const std::string& pad) {
+      auto coop_spmv = [&](int w, const std::string& first, const std::string& wfirst, const std::string& wrows,
+                           const std::string& pad) {
         for (int k = i; k < j; ++k) {
           const Task& t = S.tasks[k];
           if (t.op != DFS_OP_SPMV) continue;
           const Arg& y = t.args[4];
           const int yb = vslots(t, 4);
           const int dt = y.dtype;
-          for (int l = 0; l < w; ++l)
-            o << pad << "const " << T(dt) << " sp" << k << "_" << l << " = spmv_warp<" << T(dt) << ">("
-              << P_(t.args[0].root) << " + " << base.at(akey(t.args[0])) << ", " << P_(t.args[1].root) << " + "
-              << base.at(akey(t.args[1])) << ", " << P_(t.args[2].root) << " + " << base.at(akey(t.args[2])) << ", "
-              << P_(t.args[3].root) << " + " << base.at(akey(t.args[3])) << ", (" << base.at(akey(y)) << " - D.v["
-              << yb + 2 << "] + " << first << " + " << l << "), act_, (int)D.v[" << kslot(t) << "]);\n";
+          const std::string ops = P_(t.args[0].root) + " + " + base.at(akey(t.args[0])) + ", " + P_(t.args[1].root) + " + " +
+                                  base.at(akey(t.args[1])) + ", " + P_(t.args[2].root) + " + " + base.at(akey(t.args[2])) +
+                                  ", " + P_(t.args[3].root) + " + " + base.at(akey(t.args[3])) + ", (" + base.at(akey(y)) +
+                                  " - D.v[" + std::to_string(yb + 2) + "] + ";
+          const std::string sp = "sp" + std::to_string(k);
+          if (by_rows) {
+            o << pad << T(dt) << " " << sp << "[" << w << "];\n";
+            o << pad << "spmv_rows<" << T(dt) << ", " << w << ">(" << ops << wfirst << "), " << wrows << ", (" << T(dt)
+              << "*)(dfs_sp_raw + (threadIdx.x >> 5) * kSpmvWarpBytes), " << sp << ");\n";
+            for (int l = 0; l < w; ++l)
+              o << pad << "const " << T(dt) << " " << sp << "_" << l << " = " << sp << "[" << l << "];\n";
+          } else {
+            for (int l = 0; l < w; ++l)
+              o << pad << "const " << T(dt) << " " << sp << "_" << l << " = spmv_warp<" << T(dt) << ">(" << ops << first
+                << " + " << l << "), act_, (int)D.v[" << kslot(t) << "]);\n";
+          }
           spre[k] = "sp" + std::to_string(k);
         }
       };
@@ -450,7 +463,8 @@ void BatchGen::vector_group(int g) {
         o << ind << "  for (i64 wb = (i64)threadIdx.x - lane_; wb < nv; wb += " << BD << ") {\n";
         o << ind << "    const i64 v = wb + lane_;\n";
         o << ind << "    const bool act_ = v < nv;\n";
-        coop_spmv(V, "v * " + std::to_string(V), ind + "    ");
+        coop_spmv(V, "v * " + std::to_string(V), "wb * " + std::to_string(V),
+                  "(int)min(nv - wb, (i64)32) * " + std::to_string(V), ind + "    ");
         o << ind << "    if (act_) {\n";
         body(V, {"r"}, {"(v) * " + std::to_string(V)}, ind + "      ");
         o << ind << "    }\n";
@@ -462,7 +476,8 @@ void BatchGen::vector_group(int g) {
         o << ind << "    const i64 e = wb + lane_;\n";
       }
       o << ind << "    const bool act_ = e < n;\n";
-      coop_spmv(1, "e", ind + "    ");
+      coop_spmv(1, "e", V > 1 ? "nv * " + std::to_string(V) + " + wb" : "wb", "(int)min(n - (e - lane_), (i64)32)",
+                ind + "    ");
       o << ind << "    if (act_) {\n";
       body(1, {"t"}, {"e"}, ind + "      ");
       o << ind << "    }\n";
@@ -538,7 +553,13 @@ bool BatchGen::run(BatchCode& out, std::string& why) {
   // staging x windows needs one-row-per-lane SpMVs (no lanes shared)
   for (const Task& t : S.tasks)
     if (!coop && t.op == DFS_OP_SPMV && t.args.size() == 6) stage = true;
+  for (const Task& t : S.tasks)
+    if (!coop && !stage && t.op == DFS_OP_SPMV && t.args[4].dtype == DFS_F32) by_rows = true;
   o << "  __shared__ double red_buf[" << S.block << "];\n";
+  if (by_rows) {
+    bc.dyn_smem = S.block / 32 * kSpmvWarpBytes;
+    o << "  extern __shared__ __align__(128) unsigned char dfs_sp_raw[];\n";
+  }
   o << "  __shared__ i64 s_ticket;\n";
   o << "  Ctl* ctl = P.ctl;\n  const i64 NI = P.ninst;\n";
   if (stage) {

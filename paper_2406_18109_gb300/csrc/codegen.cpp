@@ -91,6 +91,7 @@ struct Nest {
   int vec;          // elements per vector access
   int rank = 1;     // rank of the iteration space (rows of a 3-D space are (plane, row) pairs)
   bool coop = false;  // an SpMV of the nest uses several lanes per row (spmv_warp)
+  bool rows = false;  // the nest's SpMVs are computed a warp's rows at a time (spmv_rows)
   // realigned rows: vectors in the frame of the written views (`head` scalar
   // columns first); a read view whose column origin is `shift` elements past
   // that frame is loaded as two aligned vectors
@@ -112,7 +113,6 @@ class Gen {
 
   KernelCode run();
 
- private:
   // How the loop nests of group g sweep their space (empty: several nests).
   std::string form(int g) {
     const std::vector<Nest> v = nests_of(g);
@@ -121,6 +121,7 @@ class Gen {
            std::to_string(v[0].head);
   }
 
+ private:
   const LaunchSpec& S;
   std::ostringstream o;
   KernelCode kc;
@@ -344,6 +345,8 @@ std::vector<Nest> Gen::nests_of(int g) {
     if (!aligned && vec > 1 && n.dims == 2) realign(n, vec);
     for (int t = i; t < j; ++t)
       if (S.tasks[t].op == DFS_OP_SPMV && spmv_k(S.tasks[t]) > 1) n.coop = true;
+    for (int t = i; t < j; ++t)
+      if (S.tasks[t].op == DFS_OP_SPMV && !n.coop && n.dims == 1 && S.tasks[t].args[4].dtype == DFS_F32) n.rows = true;
     v.push_back(n);
     i = j;
     while (i < G.end && S.tasks[i].scalar()) ++i;
@@ -843,27 +846,39 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
   const std::string stp = flat ? "gs" : std::to_string(BD);
   if (flat) o << ind << "  const i64 gs = (i64)gridDim.x * " << BD << ";\n";
   auto slot_off = [&](int u) { return flat ? std::to_string(u) + " * gs" : std::to_string(u * BD); };
-  if (n.dims == 1 && n.coop) {
-    // SpMV rows shared by lanes (spmv_warp).  Elements are dealt to threads
-    // exactly as in the plain loops (vectors of V in thread order, then the
+  const bool by_rows = n.rows && !stage;
+  if (n.dims == 1 && (n.coop || by_rows)) {
+    // SpMV rows shared by lanes (spmv_warp), or a warp's rows summed from
+    // shared memory (spmv_rows).  Elements are dealt to threads exactly as in
+    // the plain loops (vectors of V in thread order, then the
     // scalar tail), so reductions fused here sum in the same order; each trip
     // a warp takes 32 consecutive vectors, so all its lanes run the same trips
     o << ind << "  const i64 n = ";
     for (int d = 0; d < nd; ++d) o << (d ? " * " : "") << "ext" << d;
     o << ";\n";
     o << ind << "  const int lane_ = threadIdx.x & 31;\n";
-    auto coop_spmv = [&](int w, const std::string& first, const std::string& pad) {
+    auto coop_spmv = [&](int w, const std::string& first, const std::string& wfirst, const std::string& wrows,
+                         const std::string& pad) {
       for (int i = n.first; i < n.last; ++i) {
         const Task& t = S.tasks[i];
         if (t.op != DFS_OP_SPMV) continue;
         const Arg& y = t.args[4];
         const int dt = y.dtype;
-        for (int l = 0; l < w; ++l)
-          o << pad << "const " << T(dt) << " sp" << i << "_" << l << " = spmv_warp<" << T(dt) << ">("
-            << ptr(t.args[0].root) << " + " << base.at(akey(t.args[0])) << ", " << ptr(t.args[1].root) << " + "
-            << base.at(akey(t.args[1])) << ", " << ptr(t.args[2].root) << " + " << base.at(akey(t.args[2])) << ", "
-            << ptr(t.args[3].root) << " + " << base.at(akey(t.args[3])) << ", (" << base.at(akey(y)) << " - "
-            << y.part.vlo[0] << "LL + " << first << " + " << l << "), act_, " << spmv_k(t) << ");\n";
+        const std::string ops = ptr(t.args[0].root) + " + " + base.at(akey(t.args[0])) + ", " + ptr(t.args[1].root) + " + " +
+                                base.at(akey(t.args[1])) + ", " + ptr(t.args[2].root) + " + " + base.at(akey(t.args[2])) +
+                                ", " + ptr(t.args[3].root) + " + " + base.at(akey(t.args[3])) + ", (" + base.at(akey(y)) +
+                                " - " + std::to_string(y.part.vlo[0]) + "LL + ";
+        const std::string sp = "sp" + std::to_string(i);
+        if (by_rows) {
+          o << pad << T(dt) << " " << sp << "[" << w << "];\n";
+          o << pad << "spmv_rows<" << T(dt) << ", " << w << ">(" << ops << wfirst << "), " << wrows << ", (" << T(dt)
+            << "*)(dfs_sp_raw + (threadIdx.x >> 5) * kSpmvWarpBytes), " << sp << ");\n";
+          for (int l = 0; l < w; ++l) o << pad << "const " << T(dt) << " " << sp << "_" << l << " = " << sp << "[" << l << "];\n";
+        } else {
+          for (int l = 0; l < w; ++l)
+            o << pad << "const " << T(dt) << " " << sp << "_" << l << " = spmv_warp<" << T(dt) << ">(" << ops << first
+              << " + " << l << "), act_, " << spmv_k(t) << ");\n";
+        }
         spre[i] = "sp" + std::to_string(i);
       }
     };
@@ -872,7 +887,8 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
       o << ind << "  for (i64 wb = " << st0 << " - lane_; wb < nv; wb += " << stp << ") {\n";
       o << ind << "    const i64 v = wb + lane_;\n";
       o << ind << "    const bool act_ = v < nv;\n";
-      coop_spmv(V, "v * " + std::to_string(V), ind + "    ");
+      coop_spmv(V, "v * " + std::to_string(V), "wb * " + std::to_string(V),
+                "(int)min(nv - wb, (i64)32) * " + std::to_string(V), ind + "    ");
       o << ind << "    if (act_) {\n";
       body(V, {"r"}, {"(v) * " + std::to_string(V)}, {""}, {""}, ind + "      ");
       o << ind << "    }\n";
@@ -884,7 +900,8 @@ void Gen::emit_nest(int g, const Nest& n, const std::string& ptvar, bool flat) {
       o << ind << "    const i64 e = wb + lane_;\n";
     }
     o << ind << "    const bool act_ = e < n;\n";
-    coop_spmv(1, "e", ind + "    ");
+    coop_spmv(1, "e", V > 1 ? "nv * " + std::to_string(V) + " + wb" : "wb", "(int)min(n - (e - lane_), (i64)32)",
+              ind + "    ");
     o << ind << "    if (act_) {\n";
     body(1, {"t"}, {"e"}, {""}, {""}, ind + "      ");
     o << ind << "    }\n";
@@ -1854,6 +1871,14 @@ KernelCode Gen::run() {
     o << "  __shared__ __align__(8) u64 xs_mbar_;\n  u32 xs_ph_ = 0;\n  bool xs_live_ = true;\n";
     o << "  xstage_init(&xs_mbar_);\n";
   }
+  bool by_rows = false;
+  for (int g = 0; g < (int)S.groups.size() && !stage && !by_rows; ++g)
+    if (!S.groups[g].scalar)
+      for (const Nest& n : nests_of(g)) by_rows = by_rows || n.rows;
+  if (by_rows) {
+    kc.dyn_smem = S.block / 32 * kSpmvWarpBytes;
+    o << "  extern __shared__ __align__(128) unsigned char dfs_sp_raw[];\n";
+  }
   emit_prologue();
   for (const Group& G : S.groups)
     if (G.wave) {
@@ -1919,16 +1944,9 @@ KernelCode Gen::run() {
     }
     if (kc.nwaves) o << "      ctl->epoch = ep_ + " << kc.nwaves << "ull;\n";
     o << "    }\n";
+    o << "    ctl_reset(ctl);\n";
+    o << "  }\n";
   }
-  o << "    if (threadIdx.x == 0) {\n";
-  for (const LaunchRoot& r : S.roots) {
-    if (!r.zero_d || !r.live_out || r.param < 0) continue;
-    o << "      *" << ptr(r.root) << " = " << sreg.at(r.root) << ";\n";
-  }
-  if (kc.nwaves) o << "      ctl->epoch = ep_ + " << kc.nwaves << "ull;\n";
-  o << "    }\n";
-  o << "    ctl_reset(ctl);\n";
-  o << "  }\n";
   kc.nbarriers = nbar;
 
   std::ostringstream src;
@@ -2018,12 +2036,6 @@ void LaneOps::define(const std::string& res) {
     throw std::runtime_error("code generator: value " + res + " defined twice in one loop body");
 }
 
-KernelCode generate(const LaunchSpec& spec) {
-  Gen g(spec);
-  return g.run();
-}
-
-}  // namespace dfs
 namespace {
 
 // A task of one list writes or reduces a store that a task of the other uses.
@@ -2122,3 +2134,9 @@ void pack_groups(LaunchSpec& S) {
   S.groups = std::move(gs);
 }
 
+KernelCode generate(const LaunchSpec& spec) {
+  Gen g(spec);
+  return g.run();
+}
+
+}  // namespace dfs

@@ -394,6 +394,100 @@ __device__ __forceinline__ T spmv_warp(const int* __restrict__ rowptr, const int
   return act ? mine : T(0);
 }
 
+// y of 32 * W consecutive rows of A x, by one warp: rows row0 .. row0 + nrows
+// (nrows <= 32 * W, uniform over the warp); lane l gets rows row0 + W l + i in
+// y[i] (0 past the last row).  `buf` is the warp's own kSpmvWarpBytes of shared
+// memory.
+//
+// Bound by the L1 when every lane walks its own row: one load of col or val
+// touches a line per lane (rows of 16 entries, or W rows a lane), so a warp
+// instruction costs up to 32 tag lookups for 32 entries.  Here the rows'
+// entries, which are one contiguous run, are taken in entry order: lane q takes
+// entries q, q + 32, ..., so col and val arrive in whole lines, the gathers of
+// x of a chunk are all in flight at once, and both go to shared memory by
+// cp.async without passing through registers.  Then each lane sums its rows
+// from shared memory (rows row0 + 32 j + lane: neighbouring lanes read
+// neighbouring rows), entries in order with fma: the bits of spmv_row.
+// Row bounds that decrease (not a CSR matrix, but accepted) go row by row.
+constexpr int kSpmvWarpBytes = 2048;  // us as above at 1536 / 2048 / 4096 / 5120: 958 / 921 / 916 / 978
+template <typename T> __device__ __forceinline__ void cp_async_elem(T* s, const T* g) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((u32)__cvta_generic_to_shared(s)), "l"(g),
+               "n"(sizeof(T))
+               : "memory");
+}
+template <typename T, int W>
+__device__ __forceinline__ void spmv_rows(const int* __restrict__ rowptr, const int* __restrict__ col,
+                                          const T* __restrict__ val, const T* x, i64 row0, int nrows, T* buf,
+                                          T (&y)[W]) {
+  constexpr u32 C = kSpmvWarpBytes / (2 * sizeof(T));
+  constexpr int U = 4;
+  static_assert(C >= 32 * W, "the sums are dealt out through the buffer");
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  int k0[W], k1[W];
+#pragma unroll
+  for (int j = 0; j < W; ++j) k0[j] = __ldg(rowptr + row0 + min(32 * j + lane, nrows));
+  const int e1 = __ldg(rowptr + row0 + nrows);
+  bool mono = true;
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    const int after = __shfl_down_sync(full, k0[j], 1);
+    const int first = j + 1 < W ? __shfl_sync(full, k0[j + 1 < W ? j + 1 : j], 0) : e1;
+    k1[j] = lane < 31 ? after : first;
+    mono = mono && k1[j] >= k0[j];
+  }
+  if (!__all_sync(full, mono)) {
+#pragma unroll
+    for (int i = 0; i < W; ++i) y[i] = W * lane + i < nrows ? spmv_row<T>(rowptr, col, val, x, row0 + W * lane + i) : T(0);
+    return;
+  }
+  const int e0 = __shfl_sync(full, k0[0], 0);
+  const u32 ne = (u32)(e1 - e0);
+  T* const sv = buf;
+  T* const sx = buf + C;
+  T acc[W];
+#pragma unroll
+  for (int j = 0; j < W; ++j) acc[j] = T(0);
+  for (u32 at = 0; at < ne; at += C) {
+    const u32 m = min(C, ne - at);
+    const int* const cp = col + e0 + at;
+    const T* const vp = val + e0 + at;
+    for (u32 s = lane; s < m; s += 32 * U) {
+      int c[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (s + 32 * u < m) c[u] = __ldg(cp + s + 32 * u);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (s + 32 * u < m) cp_async_elem(sv + s + 32 * u, vp + s + 32 * u);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (s + 32 * u < m) cp_async_elem(sx + s + 32 * u, x + c[u]);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      const u32 lo = max((u32)(k0[j] - e0), at), hi = min((u32)(k1[j] - e0), at + m);
+      T a = acc[j];
+#pragma unroll 4
+      for (u32 k = lo; k < hi; ++k) a = red_fma(sv[k - at], sx[k - at], a);
+      acc[j] = a;
+    }
+    __syncwarp();
+  }
+  if (W == 1) {
+    y[0] = acc[0];
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < W; ++j) buf[32 * j + lane] = acc[j];
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < W; ++i) y[i] = buf[W * lane + i];
+  __syncwarp();
+}
+
 // ----------------------------------------------------------- control block
 // One per context, zero-initialised; every kernel leaves it zeroed on exit.
 constexpr int kTickets = 16;
@@ -800,8 +894,6 @@ template <typename T> __device__ __forceinline__ T sum_partials(const T* partial
   for (i64 i = l; i < n; i += 32) acc += ld(partials + i);
   return warp_sum_xor(acc);
 }
-
-}  // namespace dfs
 // The same sum (the same bits) with eight loads in flight per lane: every CTA
 // of a single launch waits for it between two phases.  One 0-d result of 582
 // FP64 partials took 2.3 to 6 us of a 76 us CG iteration, so 1.3 to 3.3 (CG at
@@ -823,3 +915,5 @@ template <typename T> __device__ __forceinline__ T sum_partials8(const T* partia
   }
   return warp_sum_xor(acc);
 }
+
+}  // namespace dfs

@@ -940,8 +940,6 @@ int flush_batch(dfs_ctx* c) {
   // of one-off problems of new sizes then compiles nothing new
   if (inst.empty()) return flush(c);
   if (c->cfg.launch_mode != DFS_LAUNCH_PERSISTENT || !c->cfg.fusion) return fallback("batching runs fused, persistent launches");
-  const int K = (int)inst.size();
-  std::vector<std::vector<Task>> iw(K);
   // Points are dealt in the order of the instances, and a phase ends with its
   // slowest point: those with the most entries go first, unless all have about
   // the same.  (2048 rows of about 16 scattered entries take 100 us; dealt
@@ -967,6 +965,8 @@ int flush_batch(dfs_ctx* c) {
       inst = std::move(sorted);
     }
   }
+  const int K = (int)inst.size();
+  std::vector<std::vector<Task>> iw(K);
   std::vector<std::map<int64_t, RootInfo>> iroots(K);
   std::vector<std::vector<int64_t>> canon(K);
   for (int i = 0; i < K; ++i) {

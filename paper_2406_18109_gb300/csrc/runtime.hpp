@@ -326,6 +326,7 @@ inline int spmv_lanes(int64_t nnz, int64_t nrows) {
   return k;
 }
 
+constexpr int kSpmvWarpBytes = 2048;  // shared memory of a warp for spmv_rows (dfs_device.cuh has the same)
 // Returns false (with a reason) when the launch cannot be batched.
 // coop: some instance's SpMV shares rows between lanes (spmv_lanes > 1);
 // without it SpMV nests keep one row per lane and the unrolled loops.
