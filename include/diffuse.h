@@ -278,6 +278,13 @@ int dfs_partition_tiling(dfs_ctx *ctx, int32_t ndim, const int64_t *tile, const 
 int dfs_submit(dfs_ctx *ctx, int32_t op, int32_t ndim, const int64_t *launch_domain,
                int32_t nargs, const dfs_arg *args);
 
+/* dfs_store_create, then dfs_submit with the new store as the last argument
+ * (args[nargs - 1].store is not read): one call per operator of an array
+ * expression.  When the task is refused the store is released again. */
+int dfs_submit_new(dfs_ctx *ctx, int32_t op, int32_t ndim, const int64_t *launch_domain,
+                   int32_t nargs, const dfs_arg *args, int32_t dtype, int32_t store_ndim,
+                   const int64_t *shape, dfs_store *out);
+
 /* flush_window(): analyses and launches every buffered task; asynchronous. */
 int dfs_flush(dfs_ctx *ctx);
 

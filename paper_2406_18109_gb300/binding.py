@@ -41,7 +41,7 @@ EXPORTS = ("dfs_config_default", "dfs_init", "dfs_shutdown", "dfs_store_create",
            "dfs_read_scalars_async", "dfs_record", "dfs_wait", "dfs_poll", "dfs_ticket_elapsed_ms",
            "dfs_ticket_release", "dfs_template_begin", "dfs_template_end", "dfs_template_inputs",
            "dfs_template_replay", "dfs_template_free", "dfs_rowblock_bounds", "dfs_rowblock_sizes",
-           "dfs_rowblock_plan", "dfs_spmv_windows")
+           "dfs_rowblock_plan", "dfs_spmv_windows", "dfs_submit_new")
 SPMV_STAGE_BYTES = 53248          # DFS_SPMV_STAGE_BYTES
 
 
@@ -95,6 +95,7 @@ def lib():
             "dfs_partition_none": (C.c_int, [P, pI64]),
             "dfs_partition_tiling": (C.c_int, [P, I32, pI64, pI64, C.POINTER(C.c_int32), pI64]),
             "dfs_submit": (C.c_int, [P, I32, I32, pI64, I32, C.POINTER(dfs_arg)]),
+            "dfs_submit_new": (C.c_int, [P, I32, I32, pI64, I32, C.POINTER(dfs_arg), I32, I32, pI64, pI64]),
             "dfs_flush": (C.c_int, [P]),
             "dfs_sync": (C.c_int, [P]),
             "dfs_last_error": (C.c_char_p, [P]),

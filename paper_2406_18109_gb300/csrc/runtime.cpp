@@ -1946,6 +1946,34 @@ int dfs_submit(dfs_ctx* c, int32_t op, int32_t ndim, const int64_t* dom, int32_t
   }
 }
 
+int dfs_submit_new(dfs_ctx* c, int32_t op, int32_t ndim, const int64_t* dom, int32_t nargs, const dfs_arg* args,
+                   int32_t dtype, int32_t store_ndim, const int64_t* shape, dfs_store* out) {
+  try {
+    if (!c || !out) return DFS_ERR_INVALID;
+    constexpr int kArgs = 8;
+    if (!args || nargs < 1 || nargs > kArgs) return fail(c, DFS_ERR_INVALID, "unknown op or wrong argument count");
+    dfs_store h = 0;
+    int rc = dfs_store_create(c, dtype, store_ndim, shape, &h);
+    if (rc) return rc;
+    dfs_arg a[kArgs];
+    std::copy(args, args + nargs, a);
+    a[nargs - 1].store = h;
+    rc = dfs_submit(c, op, ndim, dom, nargs, a);
+    if (rc) {
+      const std::string why = c->err;
+      dfs_store_release(c, h);
+      c->err = why;
+      return rc;
+    }
+    *out = h;
+    return DFS_OK;
+  } catch (const std::exception& e_) {
+    return internal_error(c, e_.what());
+  } catch (...) {
+    return internal_error(c, "unknown exception");
+  }
+}
+
 int dfs_flush(dfs_ctx* c) {
   try {
     if (!c) return DFS_ERR_INVALID;
