@@ -1177,6 +1177,20 @@ int Gen::emit_warp0_scalars(int g) {
 int64_t origin_of(const Arg& a, int d) { return std::max(a.part.off[d], a.part.vlo[d]); }
 int64_t floor_div(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
+// The sweeps' row and column numbers are 32-bit, sums of two of them included
+// (the last bands start up to a band past the last row): stores with a longer
+// side take the two phases, whose indices are 64-bit.
+bool sides_fit(const LaunchSpec& S, int g) {
+  for (int i = S.groups[g].begin; i < S.groups[g + 1].end; ++i)
+    for (const Arg& a : S.tasks[i].args) {
+      if (a.imm || a.nd == 0) continue;
+      const LaunchRoot& r = S.roots[S.root_index.at(a.root)];
+      for (int d = 0; d < r.ndim; ++d)
+        if (r.shape[d] >= (int64_t(1) << 30)) return false;
+    }
+  return true;
+}
+
 }  // namespace
 
 bool wave_legal(const LaunchSpec& S, int g) {
@@ -1223,7 +1237,7 @@ WaveGeom wave_geometry(const LaunchSpec& S, int g) {
     if (W.ext[d] <= 0) return W;
     elems *= W.ext[d];
   }
-  if (elems < kWaveMinElems || elems >= (int64_t(1) << 31)) return W;
+  if (elems < kWaveMinElems || elems >= (int64_t(1) << 31) || !sides_fit(S, g)) return W;
   const int cd = W.nd - 1;
   // vector width: every row of every store in memory starts on a vector
   size_t esz = 0;
@@ -1312,7 +1326,7 @@ MarchGeom march_geometry(const LaunchSpec& S, int g) {
   const Task& last = S.tasks[B.end - 1];
   M.rows = std::min(last.dom[0] * out.part.tile[0] + out.part.off[0], out.part.vhi[0]) - M.w0;
   M.cols = std::min(last.dom[1] * out.part.tile[1] + out.part.off[1], out.part.vhi[1]) - M.wc;
-  if (M.rows <= 0 || M.cols <= 0 || M.rows * M.cols < kWaveMinElems) return M;
+  if (M.rows <= 0 || M.cols <= 0 || M.rows * M.cols < kWaveMinElems || !sides_fit(S, g)) return M;
   const size_t esz = dtype_size(out.dtype);
   const int vec = (int)(16 / esz);
   M.V = X.aligned16 && X.stride[0] % vec == 0 ? vec : 1;
