@@ -1855,12 +1855,20 @@ void Gen::emit_wave(int g) {
         for (int l = 0; l < V; ++l) o << in2 << h << ".v[" << l << "] = " << vv[u * V + l] << ";\n";
     }
   }
-  o << ind << "  wave_read_done(&wsync_, wrd_ + (live ? 1u : 0u), 0u";
-  for (size_t k = 0; k < outs.size(); ++k)
+  // Every value computed from the loads, as one word.  The elements of one
+  // result are distinct cells, but two results may hold the same values (an
+  // intermediate that the application keeps and the centre it is copied to) or
+  // negated ones, so results are combined by a rotation and a sum, which do not
+  // cancel as an exclusive or of equal words does.
+  for (size_t k = 0; k < outs.size(); ++k) {
+    std::string x;
     for (int u = 0; u < Rr; ++u)
       for (int l = 0; l < V; ++l)
-        o << " ^ bits_of(n" << k << "_" << u << (V > 1 ? ".v[" + std::to_string(l) + "]" : std::string()) << ")";
-  o << ");\n";
+        x += (x.empty() ? "" : " ^ ") + std::string("bits_of(n") + std::to_string(k) + "_" + std::to_string(u) +
+             (V > 1 ? ".v[" + std::to_string(l) + "]" : std::string()) + ")";
+    o << in2 << (k == 0 ? "u32 used_ = " + x : "used_ = __funnelshift_l(used_, used_, 1) + (" + x + ")") << ";\n";
+  }
+  o << ind << "  wave_read_done(&wsync_, wrd_ + (live ? 1u : 0u), used_);\n";
   o << ind << "  }\n";
   // the previous tile's results, once every tile that reads it has read
   o << ind << "  if (live) {\n";

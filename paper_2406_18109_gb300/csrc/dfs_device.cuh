@@ -652,9 +652,11 @@ __device__ __forceinline__ bool wave_ready(WaveSync* w, u32 round, Ctl* ctl, u64
   return *(volatile int*)&w->fail == 0;
 }
 __device__ __forceinline__ void wave_pause() { asm volatile("nanosleep.u32 0;" ::: "memory"); }
-// A working warp whose loads of a tile have returned: `used` combines every
-// value computed from them, and the branch on it keeps the arrival behind the
-// loads' completion, not only behind their issue.
+// A working warp that has read a tile.  What orders its loads before a
+// neighbour's overwrite is the chain of release and acquire: its arrival on
+// `read`, the ordering warp's flag, the neighbour's poll.  On top of that
+// `used` combines every value computed from the loads (in a way that cannot
+// cancel), and the branch on it holds the arrival until they have returned.
 __device__ __forceinline__ u32 bits_of(float v) { return (u32)__float_as_int(v); }
 __device__ __forceinline__ u32 bits_of(double v) {
   const u64 b = (u64)__double_as_longlong(v);

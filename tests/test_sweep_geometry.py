@@ -1,4 +1,7 @@
 """Which form an in-place sweep takes, from the generated source (no GPU)."""
+import random
+import re
+
 import numpy as np
 import pytest
 
@@ -43,3 +46,45 @@ def test_sides_beyond_32_bit_indices_take_two_phases(shape, rows, cols, dtype):
 def test_ordinary_sides_are_swept_in_place(shape, form):
     src = _source(lambda rt: _relax(rt.empty(shape, np.float32)))
     assert (form in src) if form else "in-place sweep" not in src
+
+
+def _relax_and_keep(rt, shape, dtype, negated):
+    """The application keeps the intermediate, in views of the centre's phase."""
+    inside = tuple(slice(1, -1) for _ in shape)
+    g, kept = rt.empty(shape, dtype), rt.empty(shape, dtype)[inside]
+    acc = g[inside]
+    for d in range(len(shape)):
+        for o in (slice(0, -2), slice(2, None)):
+            acc = acc + g[tuple(o if k == d else slice(1, -1) for k in range(len(shape)))]
+    kept[...] = 0.125 * acc
+    g[inside][...] = -kept if negated else kept
+    return g, kept
+
+
+@pytest.mark.parametrize("shape", [(200, 333), (200, 336), (20, 33, 41)])
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("negated", [False, True])
+def test_the_word_of_the_values_read_does_not_cancel(shape, dtype, negated):
+    """A tile's arrival waits for a word made of all its results: it must depend
+    on them where the sweep stores one value twice, or a value and its negation."""
+    src = _source(lambda rt: _relax_and_keep(rt, shape, dtype, negated))
+    assert "in-place sweep of" in src and " bands of " not in src
+    lines = re.findall(r"u32 used_ = ([^;]*);|\n +used_ = ([^;]*);", src)
+    arg = re.search(r"wave_read_done\(&wsync_, wrd_ \+ \(live \? 1u : 0u\), (.*)\);", src).group(1)
+    names = re.findall(r"bits_of\((n\d+)(_[^)]*)\)", arg + "".join(a + b for a, b in lines))
+    assert {n for n, _ in names} == {"n0", "n1"}
+
+    def word(vals):
+        def ev(expr, used):
+            expr = re.sub(r"bits_of\(n(\d+)(_[^)]*)\)",
+                          lambda m: str(vals[m.group(2)] ^ (0x80000000 if negated and m.group(1) == "1" else 0)), expr)
+            rotl = lambda a, b, k: (a << k | b >> (32 - k)) & 0xffffffff  # noqa: E731
+            return eval(re.sub(r"\b(\d+)u\b", r"\1", expr), {"used_": used, "__funnelshift_l": rotl}) & 0xffffffff
+        used = None
+        for a, b in lines:
+            used = ev(a or b, used)
+        return ev(arg, used)
+
+    r = random.Random(1)
+    elems = {e for _, e in names}
+    assert len({word({e: r.getrandbits(32) for e in elems}) for _ in range(16)}) == 16
