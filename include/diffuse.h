@@ -169,7 +169,10 @@ typedef struct {
   const char *cache_dir;     /* on-disk cubin cache directory, or NULL */
   /* Test hook (0 = off): in generated kernels CTA 0 does not arrive at grid
    * barrier number k, so every CTA's wait runs out after barrier_timeout_s
-   * and the launch ends with DFS_ERR_BARRIER_TIMEOUT at the next dfs_sync. */
+   * and the launch ends with DFS_ERR_BARRIER_TIMEOUT at the next dfs_sync.
+   * Below zero: CTA 0 does not raise flag number -k of the context's in-place
+   * sweeps.  Numbers count from 1 over the life of the context, errors included:
+   * one per sweep of tiles, two per sweep of bands (edges read, rows stored). */
   int32_t debug_skip_arrival;
   /* 1: record CUDA events immediately around every kernel launch; the
    * per-kernel device times appear in dfs_stats_json after dfs_sync. */

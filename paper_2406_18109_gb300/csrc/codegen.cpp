@@ -166,6 +166,10 @@ class Gen {
                                                                const std::vector<std::string>& eflat,
                                                                const std::string& pad);
   void emit_wave(int g);
+  // test hook: CTA 0 withholds the context's flag number -debug_skip
+  std::string raises(const std::string& flag) const {
+    return S.debug_skip < 0 ? ", blockIdx.x != 0 || " + flag + " != " + std::to_string(-(int64_t)S.debug_skip) + "ull" : std::string();
+  }
   void emit_march(int g, int sweeps);
   std::string sweep_signature(int g) const;
   // Which tasks of nest n run two lanes per instruction in a body of w lanes
@@ -1552,7 +1556,7 @@ void Gen::emit_march(int g, int sweeps) {
   for (int k = 0; k < K; ++k)
     for (int l = 0; l < V; ++l) o << " ^ bits_of(" << sl(0, k) << (V > 1 ? ".v[" + std::to_string(l) + "]" : std::string()) << ")";
   o << ";\n" << in2 << "  if (used_ == 0x7fc5a3d1u) wave_pause(); }\n";
-  o << in2 << "march_raise(P.flags, fw);\n";
+  o << in2 << "march_raise(P.flags, fw" << raises("fw") << ");\n";
   o << in2 << "for (int n0 = 0; n0 < " << M.BR << "; n0 += " << steps << ") {\n";
   for (int u = 0; u < steps; ++u) {
     o << in2 << "  { // row ra + n0 + " << u << "\n";
@@ -1641,7 +1645,7 @@ void Gen::emit_march(int g, int sweeps) {
     o << in2 << "  }\n";
   }
   o << in2 << "}\n";
-  if (sweeps > 1) o << in2 << "if (mok && sw + 1 < " << sweeps << ") march_raise(P.flags, fw + 1);\n";
+  if (sweeps > 1) o << in2 << "if (mok && sw + 1 < " << sweeps << ") march_raise(P.flags, fw + 1" << raises("fw + 1") << ");\n";
   o << in2 << "}\n" << ind << "}\n";
   if (sweeps > 1) o << ind << "}\n";
   o << ind << "if (!mok) break;\n";
@@ -1720,7 +1724,7 @@ void Gen::emit_wave(int g) {
   for (const auto& rr : W.readers) nflag += rr.second - rr.first + 1;
   o << ind << "if (threadIdx.x >= " << BD << ") {\n";
   o << ind << "  for (i64 t = blockIdx.x; t < " << W.tiles << "LL; t += gridDim.x, ++wrd_) {\n";
-  o << ind << "    bool ok_ = wave_raise(&wsync_, wrd_, P.flags + t, ctl, fw, P.timeout_ns);\n";
+  o << ind << "    bool ok_ = wave_raise(&wsync_, wrd_, P.flags + t, ctl, fw, P.timeout_ns" << raises("fw") << ");\n";
   if (nflag > 0) {
     o << ind << "    for (int i = threadIdx.x & 31; i < " << nflag << " && ok_; i += 32) {\n";
     o << ind << "      const i64 u = t + i + (";

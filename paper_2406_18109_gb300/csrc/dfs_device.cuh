@@ -668,11 +668,12 @@ __device__ __forceinline__ void wave_read_done(WaveSync* w, u32 round, u32 used)
   if ((threadIdx.x & 31) == 0) mbar_arrive(&w->read[round & 1]);
 }
 // The ordering warp, for one tile: waits until its CTA has read it and raises
-// its flag ...
-__device__ __forceinline__ bool wave_raise(WaveSync* w, u32 round, u64* flag, Ctl* ctl, u64 want, u64 timeout_ns) {
+// its flag (unless the test hook withholds it) ...
+__device__ __forceinline__ bool wave_raise(WaveSync* w, u32 round, u64* flag, Ctl* ctl, u64 want, u64 timeout_ns,
+                                           bool raise = true) {
   const bool ok = mbar_wait(&w->read[round & 1], (round >> 1) & 1, timeout_ns);
   if (!ok) wave_error(w, ctl, want);
-  else if ((threadIdx.x & 31) == 0) wave_publish(flag, want);
+  else if (raise && (threadIdx.x & 31) == 0) wave_publish(flag, want);
   return ok;
 }
 // ... and, after polling the readers' flags, lets the tile be stored.
@@ -704,10 +705,10 @@ __device__ __forceinline__ bool march_wait(const u64* flags, i64 nb, i64 np, u64
   }
   return __syncthreads_and(ok ? 1 : 0) != 0;
 }
-// This CTA has reached a stage.
-__device__ __forceinline__ void march_raise(u64* flags, u64 stage) {
+// This CTA has reached a stage (`raise` is false under the test hook only).
+__device__ __forceinline__ void march_raise(u64* flags, u64 stage, bool raise = true) {
   __syncthreads();
-  if (threadIdx.x == 0) wave_publish(flags + blockIdx.x, stage);
+  if (raise && threadIdx.x == 0) wave_publish(flags + blockIdx.x, stage);
 }
 
 // Kernel exit: returns true in exactly one CTA -- the last to arrive -- after

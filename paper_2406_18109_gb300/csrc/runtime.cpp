@@ -1751,8 +1751,13 @@ static int check_device_error(dfs_ctx* c) {
   Ctl h;
   CUDA_OK(cudaMemcpy(&h, c->ctl, sizeof h, cudaMemcpyDeviceToHost));
   if (h.err != 0) {
-    cudaMemset(c->ctl, 0, sizeof(Ctl));  // sweep numbers start again, so the flags do too
-    if (c->flags) cudaMemset(c->flags, 0, (size_t)kWaveTilesMax * sizeof(uint64_t));
+    // Only the error is cleared.  Launches may still be queued or running: the
+    // counters are theirs, and zero after every kernel, one that gave up
+    // included.  The number of the in-place sweeps run so far has to go on,
+    // because their flags hold such numbers: started again, it would meet larger
+    // ones and let sweeps through unordered.
+    static_assert(offsetof(Ctl, err_where) == offsetof(Ctl, err) + sizeof(int32_t), "cleared together");
+    cudaMemset(&c->ctl->err, 0, sizeof(Ctl::err) + sizeof(Ctl::err_where));
     cudaDeviceSynchronize();
     if (h.err == 3)
       return fail(c, DFS_ERR_BARRIER_TIMEOUT, "an in-place sweep timed out waiting for a neighbouring tile");

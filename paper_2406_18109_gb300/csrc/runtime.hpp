@@ -173,7 +173,7 @@ struct LaunchSpec {
   int block = 256;
   int unroll = 2;
   bool persistent = false;
-  int debug_skip = 0;  // test hook: CTA 0 withholds its arrival at this barrier
+  int debug_skip = 0;  // test hook: CTA 0 withholds its arrival at this barrier (< 0: a sweep's flag)
   int min_blocks = 0;  // > 0: __launch_bounds__ minimum resident CTAs per SM (caps registers)
   int sms = 152;       // SMs of the device (co-resident CTAs of an in-place sweep)
 };
