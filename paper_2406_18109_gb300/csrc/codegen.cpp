@@ -1526,12 +1526,13 @@ void Gen::emit_march(int g, int sweeps) {
   }
   o << in2 << "}\n";
   if (pan) {
-    // columns: element e of the vector before (after) the panel, rows -1 .. BR
+    // columns: element e of the vector before (after) the panel, rows -1 .. BR,
+    // by the threads that own vectors (a panel is one group; the others have no rows)
     for (const auto& kv : eidx) {
       const int dv = kv.first.first, e = kv.first.second;
       const std::string v = dv < 0 ? "pb - 1" : "pb + " + std::to_string(M.PC);
       o << in2 << "if (" << v << " >= 0 && " << v << " < " << M.NC << ")\n";
-      o << in2 << "  for (int i = threadIdx.x; i < rz - ra + 2; i += " << BD << ") mp" << sfx << "[" << kv.second * (M.BR + 2)
+      o << in2 << "  for (int i = threadIdx.x; i < rz - ra + 2; i += " << M.GT << ") mp" << sfx << "[" << kv.second * (M.BR + 2)
         << " + i] = ld(" << ptr(out->root) << " + (i64)min(max(ra - 1 + i + " << M.w0 << ", 0), " << X.shape[0] - 1 << ") * " << X.stride[0] << "LL + (i64)(" << v << " + "
         << M.pv0 << ") * " << V << " + " << e << ");\n";
     }

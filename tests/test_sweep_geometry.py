@@ -88,3 +88,17 @@ def test_the_word_of_the_values_read_does_not_cancel(shape, dtype, negated):
     r = random.Random(1)
     elems = {e for _, e in names}
     assert len({word({e: r.getrandbits(32) for e in elems}) for _ in range(16)}) == 16
+
+
+@pytest.mark.parametrize("shape, kw", [((17400, 10400), {}), ((43000, 4104), dict(block=1024, unroll=1)),
+                                       ((30000, 8232), dict(block=512))], ids=str)
+def test_edge_columns_of_a_panel_are_read_whole(shape, kw):
+    """Rows of several panels: the columns next to a panel, all rows of a band,
+    are read by the threads that own vectors (fewer than the CTA's)."""
+    src = _source(lambda rt: _relax(rt.empty(shape, np.float32)), **kw)
+    rows, = re.findall(r" bands of (\d+) rows", src)
+    own, = set(re.findall(r"grp < 1 && q < (\d+)", src))
+    loops = set(re.findall(r"i < rz - ra \+ 2; i \+= (\d+)\)", src))
+    assert len(loops) == 1
+    seen = {i for q in range(int(own)) for i in range(q, int(rows) + 2, int(*loops))}
+    assert seen == set(range(int(rows) + 2))
