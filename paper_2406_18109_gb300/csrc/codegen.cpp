@@ -20,6 +20,7 @@
 // source; pointers and immediate values are kernel parameters, so isomorphic
 // windows share one compiled kernel (Section 5.2).
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <functional>
 #include <sstream>
@@ -1229,6 +1230,76 @@ bool wave_legal(const LaunchSpec& S, int g) {
   return cut;
 }
 
+namespace {
+
+// Arithmetic operations per element of a pair of groups, in units of an
+// addition (copies and signs cost no arithmetic).
+double pair_ops(const LaunchSpec& S, int g) {
+  double n = 0.0;
+  for (int i = S.groups[g].begin; i < S.groups[g + 1].end; ++i) {
+    const int op = S.tasks[i].op;
+    if (op == DFS_OP_COPY || op == DFS_OP_NEG || op == DFS_OP_ABS) continue;
+    n += op == DFS_OP_DIV || op == DFS_OP_SQRT ? 10.0 : op >= DFS_OP_ADD && op != DFS_OP_POW ? 1.0 : 25.0;
+  }
+  return n;
+}
+
+// What one sweep takes, in microseconds, as fitted to GB300 measurements (the
+// 5-point stencil of 66^2 to 8190^2 points, tall and wide grids, one, five and
+// nine operations a point, 128 to 1024 threads; within about 10 % of them).
+// The forms are compared by these estimates only, so results do not depend on
+// them: every form leaves the same bits.
+//
+// Two phases: a barrier and two flat sweeps; FP32 by L2 and HBM, FP64 by the
+// FP64 pipe, which a flat sweep keeps busy on all SMs.
+double phases_us(const LaunchSpec& S, double elems, int esz, double ops, int nd) {
+  if (esz == 4) return 6.0 + elems / 0.48e6;
+  const double pipe = elems / S.sms * (0.00045 + 0.00027 * ops);
+  return nd == 3 ? std::max(std::min(10.0, 6.0 + elems / 8192.0), 7.5 + pipe) : std::max(S.block >= 1024 ? 11.0 : 9.0, 5.5 + pipe);
+}
+// Bands: the CTA's flags, then a row of the band at a time.  FP32: a row costs
+// a round trip to L2, or what its vectors take.  FP64: the schedulers share the
+// FP64 units in such a way that a row costs as if part of the warps were
+// rounded up to eight (measured: 5, 6, 7, 8 warps 1.6, 1.7, 1.9, 2.0; 9, 10,
+// 12, 14, 16 warps 3.1, 3.3, 3.5, 3.8, 4.0 times what a warp per scheduler
+// should), whatever lanes are active: narrow rows waste it.
+double bands_us(const LaunchSpec& S, const MarchGeom& M, int esz, double ops) {
+  if (esz == 4)
+    return 4.0 + M.BR * std::max(0.22, 0.03 * ops * M.K * std::pow(S.block / 256.0, 0.6) * (1.0 + 0.05 * std::max(0, M.K - 6))) *
+                     (M.PN > 1 ? 1.3 : 1.0);
+  const int w = M.GT * M.G / 32 * std::max(1, S.min_blocks);
+  const double busy = w <= 4 ? 1.1 : w / 8.0 + (w + 7) / 8;
+  const double row = busy * M.K * (0.066 + 0.002 * ops) * ops * ((double)M.rows * M.cols * esz > 96e6 ? 1.12 : 1.0);
+  return 4.5 + M.BR * std::max(0.8, row);
+}
+
+// Tiles: a CTA's first tile, then what the FP64 pipe takes for the tiles of the
+// busiest SM (whole rounds of the resident CTAs once there are more tiles).
+double tiles_us(const LaunchSpec& S, const WaveGeom& W, double elems, double ops) {
+  const int64_t resident = (int64_t)W.min_blocks * S.sms;
+  const double q = W.tiles <= resident ? (double)((W.tiles + S.sms - 1) / S.sms)
+                                       : (double)((W.tiles + resident - 1) / resident) * W.min_blocks;
+  const double us = 6.0 + q * (S.block - 32) * W.R * W.V * 0.000311 * ops;
+  return W.nd == 2 && elems * 8 > 96e6 ? 1.15 * us : us;
+}
+// Whether tiles are below the two phases (us a sweep, tiles against phases).
+// Their polling and their rounds cost more than the barrier saves but for small
+// sweeps, where a tile is all that an SM has (5 x 10002 FP32 4.1 against 5.8;
+// 34^3 FP32 5.7 against 6.7), and for 3-D grids of one result, whose planes a
+// tile keeps in L1 (251^3 FP32 42 against 63, FP64 240 against 258).  With a
+// second result in memory (200^3 FP32 31.5 against 22.5), lines much longer than
+// a tile (48 x 48 x 2000 FP64 85 against 81) or readers most of a round away
+// (20 x 500 x 500 FP64 125 against 81) they are slower.
+bool tiles_pay(const LaunchSpec& S, const WaveGeom& W, double elems, int esz, double ops, int results) {
+  const int64_t BD = S.block - 32, resident = (int64_t)W.min_blocks * S.sms;
+  const bool small = W.tiles * 3 * std::max(1, S.block / 256) <= (int64_t)S.sms * 2;
+  if (!small && ((W.nd == 3 && W.nvx > 2 * BD) || W.reach * 3 > resident * 2)) return false;
+  if (esz == 8) return W.us + (small ? 0.0 : 0.3 * (results - 1)) < phases_us(S, elems, esz, ops, W.nd);
+  return small || (W.nd == 3 && results == 1 && elems >= (1 << 21));
+}
+
+}  // namespace
+
 WaveGeom wave_geometry(const LaunchSpec& S, int g) {
   WaveGeom W;
   const Group &A = S.groups[g], &B = S.groups[g + 1];
@@ -1314,7 +1385,15 @@ WaveGeom wave_geometry(const LaunchSpec& S, int g) {
   // less than a grid ahead (or every tile has a CTA of its own)
   W.min_blocks = S.min_blocks > 0 ? S.min_blocks : std::max(1, 1024 / S.block);
   const int64_t resident = (int64_t)W.min_blocks * S.sms;
-  W.ok = W.tiles <= resident || W.reach < resident;
+  std::set<int64_t> results;
+  for (int i = A.begin; i < B.end; ++i) {
+    const Arg& a = S.tasks[i].args.back();
+    if (!S.roots[S.root_index.at(a.root)].temp) results.insert(a.root);
+  }
+  const double ops = pair_ops(S, g);
+  W.us = tiles_us(S, W, (double)elems, ops);
+  W.ok = (W.tiles <= resident || W.reach < resident) &&
+         tiles_pay(S, W, (double)elems, (int)esz, ops, (int)results.size());
   return W;
 }
 
@@ -1364,29 +1443,47 @@ MarchGeom march_geometry(const LaunchSpec& S, int g) {
   const int64_t words = M.V * (int64_t)esz / 4, 
                 avail = std::min<int64_t>(255, 65536 / (S.block * std::max(1, S.min_blocks))) - 44;
   const int64_t kmax = avail / (words * 5);  // three rows around the computed one and two ahead
-  if (kmax < 1) return M;
-  const int64_t want = (M.NC + S.block - 1) / S.block;
-  M.PN = (want + kmax - 1) / kmax;
-  const int64_t per = (M.NC + M.PN - 1) / M.PN;
-  M.K = (int)((per + S.block - 1) / S.block);
-  M.GT = (int)(((per + M.K - 1) / M.K + 31) / 32 * 32);
-  M.PC = (int64_t)M.K * M.GT;
-  M.PN = (M.NC + M.PC - 1) / M.PC;
-  M.G = M.PN > 1 ? 1 : S.block / M.GT;
   const int64_t per_sm = S.min_blocks > 0 ? S.min_blocks : 1;
-  const int64_t ctas = std::max<int64_t>(1, per_sm * S.sms / M.PN);
-  if (M.PN > per_sm * S.sms) return M;
-  M.BR = (M.rows + ctas * M.G - 1) / (ctas * M.G);
-  M.NB = ((M.rows + M.BR - 1) / M.BR + M.G - 1) / M.G;
-  M.D = (int)std::min<int64_t>({6, avail / (words * M.K) - 3, M.BR});
   // static shared memory: the row below the band, the warps' edge elements
-  // and, between panels, the neighbours' edge columns
-  const int64_t smem = (int64_t)M.K * S.block * M.V * esz + (3 + M.D) * (int64_t)edges.size() * M.K * (S.block / 32) * esz +
-                       (M.PN > 1 ? (M.BR + 2) * (int64_t)edges.size() * esz : 0);
-  M.smem = smem;
-  if (smem > 40 * 1024 || M.NB * M.PN > kWaveTilesMax) return M;
-  M.ok = true;
-  return M;
+  // and, between panels, the neighbours' edge columns; 48 KB less the kernel's
+  // other arrays (the sums' buffer, broadcast slots)
+  const int64_t limit = std::min<int64_t>(40 * 1024, 48 * 1024 - 8 * S.block - 1024);
+  // vectors per thread: the fewest leave threads and warps of the last vector
+  // idle, the most leave too few bands; taken by the estimate above, and only
+  // where it is below that of the two phases.  Bands against two phases, us a
+  // sweep: 1000002 x 5 FP64 659 -> 49, 200002 x 34 FP32 43 -> 20 (two phases
+  // again); 20002 x 302 FP32 17.4 -> 11.3, 302 x 20002 FP32 16.6 -> 11.8 (other K).
+  const double ops = pair_ops(S, g);
+  double best = phases_us(S, (double)M.rows * M.cols, (int)esz, ops, 2);
+  if (esz == 8) {
+    const WaveGeom W = wave_geometry(S, g);
+    if (W.ok) best = std::min(best, W.us);
+  }
+  MarchGeom pick;
+  for (int64_t k = kmax; k >= 1; --k) {
+    MarchGeom C = M;
+    C.PN = (C.NC + S.block * k - 1) / (S.block * k);
+    const int64_t per = (C.NC + C.PN - 1) / C.PN;
+    C.K = (int)std::max(std::min(k, (per + 31) / 32), (per + S.block - 1) / S.block);
+    C.GT = (int)(((per + C.K - 1) / C.K + 31) / 32 * 32);
+    C.PC = (int64_t)C.K * C.GT;
+    C.PN = (C.NC + C.PC - 1) / C.PC;
+    C.G = C.PN > 1 ? 1 : S.block / C.GT;
+    const int64_t ctas = std::max<int64_t>(1, per_sm * S.sms / C.PN);
+    if (C.PN > per_sm * S.sms) continue;
+    C.BR = (C.rows + ctas * C.G - 1) / (ctas * C.G);
+    C.NB = ((C.rows + C.BR - 1) / C.BR + C.G - 1) / C.G;
+    C.D = (int)std::min<int64_t>({6, avail / (words * C.K) - 3, C.BR});
+    C.smem = (int64_t)C.K * C.GT * C.G * C.V * esz + (3 + C.D) * (int64_t)edges.size() * C.K * (C.GT * C.G / 32) * esz +
+             (C.PN > 1 ? (C.BR + 2) * (int64_t)edges.size() * esz : 0);
+    if (C.smem > limit || C.NB * C.PN > kWaveTilesMax) continue;
+    const double us = bands_us(S, C, (int)esz, ops);
+    if (us >= best) continue;
+    pick = C;
+    pick.ok = true;
+    best = us;
+  }
+  return pick;
 }
 
 namespace {
@@ -1397,7 +1494,7 @@ namespace {
 void Gen::emit_march(int g, int sweeps) {
   const MarchGeom M = march_geometry(S, g);
   const Group &A = S.groups[g], &B = S.groups[g + 1];
-  const int BD = S.block, V = M.V, K = M.K, RS = 3 + M.D, NW = BD / 32;
+  const int BD = S.block, V = M.V, K = M.K, RS = 3 + M.D, AT = M.GT * M.G, NW = AT / 32;  // AT: threads that own vectors
   const int steps = (int)std::min<int64_t>(RS, M.BR);  // rows per trip of the unrolled row loop
   Nest n;
   n.first = A.begin;
@@ -1462,7 +1559,7 @@ void Gen::emit_march(int g, int sweeps) {
   const int nimm = (kc.nimm - imm0) / sweeps;
   const bool pan = M.PN > 1 && NE;
   o << ind << T1 << "* const mb" << sfx << " = (" << T1 << "*)march_raw;  // the row below the band\n";
-  if (NE) o << ind << T1 << "* const me" << sfx << " = mb" << sfx << " + " << K * BD * V << ";  // edge elements of the warps' vectors\n";
+  if (NE) o << ind << T1 << "* const me" << sfx << " = mb" << sfx << " + " << K * AT * V << ";  // edge elements of the warps' vectors\n";
   if (pan) o << ind << T1 << "* const mp" << sfx << " = me" << sfx << " + " << RS * NE * K * NW << ";  // edge columns of the next panels\n";
   o << ind << "bool mok = true;\n";
   const std::string sw = sweeps > 1 ? "sw" : "0";
@@ -1490,7 +1587,12 @@ void Gen::emit_march(int g, int sweeps) {
     << "u + grp) * " << M.BR << ", " << M.rows << ") : " << M.rows << ", rz = min(ra + " << M.BR << ", " << M.rows << ");\n";
   o << in2 << "const bool act = ra < rz;\n";
   o << in2 << "const int pb = (int)(blockIdx.x % " << M.PN << "u) * " << M.PC << ";\n";
+  // The warp's number comes through a shuffle: with it written in place NVRTC
+  // 13.0 turned (threadIdx.x >> 5) * K + k, where only lane 31 gets there, K is
+  // a power of two and a CTA has several groups, into the address of K - 1
+  // elements further on.
   o << in2 << "const int lane = threadIdx.x & 31, lw = q >> 5;\n";
+  o << in2 << "const int wid = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);\n";
   // one warp's vectors k are consecutive; vectors past the row repeat its last
   for (int k = 0; k < K; ++k) {
     o << in2 << "const int c" << k << " = pb + " << k * M.GT << " + q;\n";
@@ -1514,7 +1616,7 @@ void Gen::emit_march(int g, int sweeps) {
     for (int k = 0; k < K; ++k) o << in3 << "  " << sl(j, k) << " = " << ldv << "(" << row_at(k, "ra + " + std::to_string(j - 1)) << ");\n";
     o << in3 << "}\n";
   }
-  auto below = [&](int k) { return "mb" + sfx + " + (" + std::to_string(k * BD) + " + threadIdx.x) * " + std::to_string(V); };
+  auto below = [&](int k) { return "mb" + sfx + " + (" + std::to_string(k * AT) + " + threadIdx.x) * " + std::to_string(V); };
   for (int k = 0; k < K; ++k) {
     if (V > 1) o << in3 << stv << "(" << below(k) << ", b" << k << ");\n";
     else o << in3 << "*(" << below(k) << ") = b" << k << ";\n";
@@ -1543,7 +1645,7 @@ void Gen::emit_march(int g, int sweeps) {
       const int dv = kv.first.first, e = kv.first.second;
       o << pad << "if (lane == " << (dv < 0 ? 31 : 0) << " && act) {";
       for (int k = 0; k < K; ++k)
-        o << " me" << sfx << "[" << (slot * NE + kv.second) * K * NW << " + (threadIdx.x >> 5) * " << K << " + " << k << "] = " << sl(j, k)
+        o << " me" << sfx << "[" << (slot * NE + kv.second) * K * NW << " + wid * " << K << " + " << k << "] = " << sl(j, k)
           << (V > 1 ? ".v[" + std::to_string(e) + "]" : std::string()) << ";";
       o << " }\n";
     }
@@ -1588,7 +1690,7 @@ void Gen::emit_march(int g, int sweeps) {
         // (after), or, past the group's last warp, in the next k
         const int base = (slot * NE + ei) * K * NW;
         const int wg = M.GT / 32;
-        const std::string w = "(int)(threadIdx.x >> 5)";
+        const std::string w = "wid";
         o << in3 << "if (lane == " << (dv > 0 ? 31 : 0) << " && act) {\n";
         const std::string at = "me" + sfx + "[" + std::to_string(base) + " + ";
         std::string panel = pan ? "mp" + sfx + "[" + std::to_string(ei * (M.BR + 2)) + " + i - ra + " + std::to_string(1 + d0) + "]" : "";

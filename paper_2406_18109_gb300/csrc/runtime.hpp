@@ -197,6 +197,7 @@ struct WaveGeom {
   std::vector<std::pair<int64_t, int64_t>> readers;  // ranges of u - t over the tiles u that read tile t
   int64_t reach = 0;                       // largest |u - t|
   int min_blocks = 1;                      // CTAs per SM the kernel is compiled to keep resident
+  double us = 0.0;                         // estimated time of an FP64 sweep
 };
 // Legality (dependences of the tasks, one shared iteration space) of running
 // groups g and g+1 of the launch as a wave.

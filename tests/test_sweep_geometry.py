@@ -42,7 +42,7 @@ def test_sides_beyond_32_bit_indices_take_two_phases(shape, rows, cols, dtype):
     assert "in-place sweep" not in src and "grid_barrier(ctl" in src
 
 
-@pytest.mark.parametrize("shape, form", [((66, 66), " bands of "), ((2 ** 30 - 1, 3), " bands of "), ((65, 65), None)])
+@pytest.mark.parametrize("shape, form", [((66, 66), " bands of "), ((2 ** 30 - 1, 3000), " bands of "), ((65, 65), None)])
 def test_ordinary_sides_are_swept_in_place(shape, form):
     src = _source(lambda rt: _relax(rt.empty(shape, np.float32)))
     assert (form in src) if form else "in-place sweep" not in src
@@ -61,7 +61,7 @@ def _relax_and_keep(rt, shape, dtype, negated):
     return g, kept
 
 
-@pytest.mark.parametrize("shape", [(200, 333), (200, 336), (20, 33, 41)])
+@pytest.mark.parametrize("shape", [(200, 333), (200, 336), (34, 34, 35)])
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
 @pytest.mark.parametrize("negated", [False, True])
 def test_the_word_of_the_values_read_does_not_cancel(shape, dtype, negated):
@@ -102,3 +102,29 @@ def test_edge_columns_of_a_panel_are_read_whole(shape, kw):
     assert len(loops) == 1
     seen = {i for q in range(int(own)) for i in range(q, int(rows) + 2, int(*loops))}
     assert seen == set(range(int(rows) + 2))
+
+
+def _seven(g):
+    c = g[1:-1, 1:-1, 1:-1]
+    acc = c + g[:-2, 1:-1, 1:-1] + g[2:, 1:-1, 1:-1] + g[1:-1, :-2, 1:-1] + g[1:-1, 2:, 1:-1] + g[1:-1, 1:-1, :-2] + g[1:-1, 1:-1, 2:]
+    work = (1.0 / 7) * acc
+    c[...] = work
+
+
+@pytest.mark.parametrize("program, shape, dtype, form", [
+    # narrow rows leave most lanes of a band idle
+    ("relax", (1000002, 5), np.float32, None), ("relax", (1000002, 5), np.float64, None),
+    ("relax", (200002, 34), np.float32, None), ("relax", (200002, 34), np.float64, None),
+    # a second result in memory, FP32
+    ("keep", (2050, 2050), np.float32, None), ("keep", (200, 200, 200), np.float32, None),
+    # readers nearly a round away; short rows that waste lanes, FP64
+    ("seven", (22, 502, 502), np.float64, None), ("seven", (502, 502, 22), np.float64, None),
+    # where they are faster: bands (with several groups of warps, with panels), tiles
+    ("relax", (8192, 8192), np.float32, " bands of "), ("relax", (20002, 302), np.float32, " bands of "),
+    ("relax", (302, 20002), np.float32, " bands of "), ("relax", (1023, 1149), np.float64, " bands of "),
+    ("seven", (253, 253, 253), np.float32, " tiles"), ("seven", (253, 253, 253), np.float64, " tiles"),
+], ids=str)
+def test_sweeps_are_in_place_where_that_is_faster(program, shape, dtype, form):
+    src = _source(lambda rt: _relax_and_keep(rt, shape, dtype, False) if program == "keep"
+                  else (_relax if program == "relax" else _seven)(rt.empty(shape, dtype)))
+    assert ("in-place sweep" in src and form in src) if form else "in-place sweep" not in src
