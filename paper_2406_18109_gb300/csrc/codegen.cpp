@@ -101,6 +101,29 @@ struct Nest {
   std::map<std::string, int> shift;
 };
 
+// Whether an FP32 SpMV's rows are computed a warp's rows at a time (spmv_rows)
+// or one per lane (spmv_row); the bits are the same.  spmv_rows wins as a rule
+// (1M rows of 7 entries 58 -> 38 us, of 31 253 -> 160) and by far where rows
+// differ in length, but not
+//  * for rows of one entry over several million rows, nothing to coalesce (4M
+//    rows: 18.0 us a lane each, 21.1 a warp's at a time);
+//  * for a few points of long rows: a warp's chunks come one after another (40000
+//    rows of 31 entries in 157 points 18.8, 21.8);
+//  * in CTAs of more than 256 threads, whose registers (48 against 32) leave half
+//    as many CTAs per SM, when the points then take another round and keep few
+//    warps busy (100000 rows of 31 in 391 points, 512 threads 26, 41), at 1024
+//    threads also for short rows (1M rows of 5 18.6, 22.0; of 16 133, 93).
+bool rows_pay(const Task& t, int block, int sms) {
+  const Arg& y = t.args[4];
+  if (y.dtype != DFS_F32) return false;
+  const int64_t nnz = t.args[1].part.vhi[0] - t.args[1].part.vlo[0], points = t.npoints();
+  const int64_t rows = t.args[0].part.vhi[0] - t.args[0].part.vlo[0] - 1, tile = y.part.kind == 1 ? y.part.tile[0] : rows;
+  if (rows >= (1 << 21) && nnz < 2 * rows) return false;
+  if (points * 4 <= sms * 5 && nnz >= 24 * rows && rows > 0) return false;
+  if (block <= 256 || points * block <= (int64_t)sms * 1024) return true;
+  return tile >= block && (block < 1024 || nnz >= 8 * rows);
+}
+
 // Lanes per row of an SpMV task's matrix (col and rowptr extents).
 int spmv_k(const Task& t) {
   const NPart& c = t.args[1].part;
@@ -356,7 +379,7 @@ std::vector<Nest> Gen::nests_of(int g) {
     for (int t = i; t < j; ++t)
       if (S.tasks[t].op == DFS_OP_SPMV && spmv_k(S.tasks[t]) > 1) n.coop = true;
     for (int t = i; t < j; ++t)
-      if (S.tasks[t].op == DFS_OP_SPMV && !n.coop && n.dims == 1 && S.tasks[t].args[4].dtype == DFS_F32) n.rows = true;
+      if (S.tasks[t].op == DFS_OP_SPMV && !n.coop && n.dims == 1 && rows_pay(S.tasks[t], S.block, S.sms)) n.rows = true;
     v.push_back(n);
     i = j;
     while (i < G.end && S.tasks[i].scalar()) ++i;
