@@ -575,27 +575,44 @@ int build_window(dfs_ctx* c, const WindowInfo& wi, std::unique_ptr<CachedWindow>
     // In-place sweeps need their CTAs resident together; where the built
     // kernel does not reach the residency the geometry counted on (a
     // ctas_per_sm beyond what shared memory or threads allow), the launch is
-    // generated again with two phases per sweep.
-    for (const bool waves : {true, false}) {
-      spec = make_spec(c, w, wi.roots, P, g0, g1, valid, waves);
+    // generated again with two phases per sweep.  Joined FP64 sweeps whose
+    // registers cost the kernel a second round of points go apart again (sums
+    // and quotients of 8M elements: 601 points, 74 registers against 64, 250
+    // against 191 us; FP32 sweeps are bound by memory and stay joined).
+    for (const bool packing : {true, false}) {
+      LaunchSpec sp = make_spec(c, w, wi.roots, P, g0, g1, valid, packing);
+      KernelCode k2;
       try {
-        kc = generate(spec);
+        k2 = generate(sp);
       } catch (const std::exception& e) {
         return fail(c, DFS_ERR_INVALID, std::string("code generation: ") + e.what());
       }
       std::string err;
-      c->last_source = kc.source;
+      const Compiled* built = nullptr;
       if (!c->device) {
         // analysis-only context: check that the kernel compiles for the target
-        if (!c->jit->compile_only(kc.source, kc.name, err)) return fail(c, DFS_ERR_COMPILE, err);
-        break;
+        c->last_source = k2.source;
+        if (!c->jit->compile_only(k2.source, k2.name, err)) return fail(c, DFS_ERR_COMPILE, err);
+      } else {
+        built = c->jit->get(k2.source, k2.name, sp.block, err, k2.dyn_smem);
+        if (!built) return fail(c, DFS_ERR_COMPILE, err);
       }
-      comp = c->jit->get(kc.source, kc.name, spec.block, err, kc.dyn_smem);
-      if (!comp) return fail(c, DFS_ERR_COMPILE, err);
-      if (kc.nwaves == 0) break;
       const int64_t resident =
-          (int64_t)(c->cfg.ctas_per_sm > 0 ? std::min(comp->occupancy, c->cfg.ctas_per_sm) : comp->occupancy) * c->sms;
-      if (kc.march_ctas <= resident && (kc.wave_tiles <= resident || kc.wave_reach < resident)) break;
+          !built ? 0 : (int64_t)(c->cfg.ctas_per_sm > 0 ? std::min(built->occupancy, c->cfg.ctas_per_sm) : built->occupancy) * c->sms;
+      // (the second variant is the joined one's alternative, taken if it fits)
+      if (!packing && kc.nwaves == 0 && k2.max_points > resident) break;
+      const bool joined = !sp.order.empty();
+      spec = std::move(sp);
+      kc = std::move(k2);
+      comp = built;
+      c->last_source = kc.source;
+      if (!built) break;
+      if (kc.nwaves > 0) {
+        if (kc.march_ctas <= resident && (kc.wave_tiles <= resident || kc.wave_reach < resident)) break;
+        continue;
+      }
+      const bool fp64 = std::any_of(spec.roots.begin(), spec.roots.end(), [](const LaunchRoot& r) { return !r.zero_d && r.dtype == DFS_F64; });
+      if (!joined || !fp64 || !kc.has_points || kc.max_points <= resident) break;
     }
     for (const LaunchRoot& lr : spec.roots)
       if (lr.param >= 0) need_mem.insert(lr.root);
