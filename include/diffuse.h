@@ -300,6 +300,9 @@ const char *dfs_last_error(dfs_ctx *ctx);
 /* JSON description of how the buffered window would be fused, without
  * launching it: {"groups": [[task indices]...], "temporaries": [store ids],
  * "launches": [[group indices]...], "barriers": n, "key": "..."}.
+ * "barriers" counts the grid barriers of the kernels the flush launches: at most
+ * one after every group that is not scalar, fewer where sweeps are joined or run
+ * in place (once the form has been flushed, of the kernels that were built).
  * Writes at most len bytes (NUL-terminated) and the full size to *needed. */
 int dfs_plan_json(dfs_ctx *ctx, char *buf, size_t len, size_t *needed);
 

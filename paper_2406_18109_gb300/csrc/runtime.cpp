@@ -378,7 +378,7 @@ WindowInfo window_info(dfs_ctx* c) {
   return wi;
 }
 
-std::string plan_json(const Plan& p, const std::vector<Task>& w, const WindowInfo& wi) {
+std::string plan_json(const Plan& p, const std::vector<Task>& w, const WindowInfo& wi, int64_t bars) {
   std::ostringstream o;
   o << "{\"groups\": [";
   for (size_t g = 0; g < p.groups.size(); ++g) {
@@ -413,10 +413,6 @@ std::string plan_json(const Plan& p, const std::vector<Task>& w, const WindowInf
     for (int g = p.launches[l].first; g < p.launches[l].second; ++g) o << (g > p.launches[l].first ? ", " : "") << g;
     o << "]";
   }
-  int bars = 0;
-  for (const auto& L : p.launches)
-    for (int g = L.first + 1; g < L.second; ++g)
-      if (!p.groups[g - 1].scalar) ++bars;
   o << "], \"scalar_groups\": [";
   first = true;
   for (size_t g = 0; g < p.groups.size(); ++g)
@@ -656,6 +652,31 @@ int build_window(dfs_ctx* c, const WindowInfo& wi, std::unique_ptr<CachedWindow>
     if (kv.second && need_mem.count(kv.first)) cw->made_valid.push_back(wi.canon.at(kv.first));
   out = std::move(cw);
   return DFS_OK;
+}
+
+// Grid barriers of the kernels a flush of the window launches: those of the
+// launches already built for this form, else of the kernels as they would be
+// generated (joined sweeps, in-place sweeps).
+int64_t window_barriers(dfs_ctx* c, const WindowInfo& wi, const Plan& P) {
+  int64_t bars = 0;
+  auto it = c->wcache.find(wi.key);
+  if (it != c->wcache.end() && it->second->launches.size() == P.launches.size()) {
+    for (const CachedLaunch& L : it->second->launches) bars += L.nbarriers;
+    return bars;
+  }
+  std::map<int64_t, bool> valid;
+  for (const auto& kv : wi.roots) valid[kv.first] = kv.second.valid;
+  for (const auto& L : P.launches) {
+    const LaunchSpec spec = make_spec(c, c->window, wi.roots, P, L.first, L.second, valid, true);
+    try {
+      bars += generate(spec).nbarriers;
+    } catch (const std::exception&) {  // a form that a flush refuses: the plan's cuts
+      for (int g = L.first + 1; g < L.second; ++g) bars += P.groups[g - 1].scalar ? 0 : 1;
+    }
+    for (const LaunchRoot& lr : spec.roots)
+      if (lr.written && lr.param >= 0) valid[lr.root] = true;
+  }
+  return bars;
 }
 
 // The flag array of in-place sweeps: fixed size, so graphs that recorded its
@@ -2562,7 +2583,7 @@ int dfs_plan_json(dfs_ctx* c, char* buf, size_t len, size_t* needed) {
     if (!c) return DFS_ERR_INVALID;
     WindowInfo wi = window_info(c);
     Plan p = analyse(c->window, wi.roots, c->cfg.fusion != 0, c->cfg.launch_mode);
-    std::string s = plan_json(p, c->window, wi);
+    std::string s = plan_json(p, c->window, wi, window_barriers(c, wi, p));
     s.insert(s.size() - 1, ", \"key\": \"" + std::to_string(std::hash<std::string>{}(wi.key)) + "\"");
     return write_json(s, buf, len, needed);
   } catch (const std::exception& e_) {
