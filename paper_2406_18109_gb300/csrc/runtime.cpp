@@ -104,6 +104,7 @@ struct dfs_ctx {
     int64_t launches = 0;
   };
   std::map<int64_t, GraphRec> graphs;
+  std::vector<void*> retired;           // scratch replaced by a larger one while graphs that recorded it live
   // batched execution
   bool batching = false;
   std::vector<size_t> batch_marks;      // window positions where instances end
@@ -205,6 +206,26 @@ void maybe_free(dfs_ctx* c, int64_t root) {
   }
   c->captured_allocs.erase(root);
   c->stores.erase(it);
+}
+
+// Scratch (partials, batch scalars) of at least `bytes`.  Graphs recorded the
+// address of the block they were captured with: while there are graphs, the old
+// block is kept for their replays and given back with the last of them.
+int grow_scratch(dfs_ctx* c, void** p, size_t* cap, size_t bytes) {
+  if (bytes <= *cap) return DFS_OK;
+  void* n = nullptr;
+  CUDA_OK(cudaMallocAsync(&n, bytes, c->stream));
+  if (*p) {
+    if (c->graphs.empty()) cudaFreeAsync(*p, c->stream);
+    else c->retired.push_back(*p);
+  }
+  *p = n;
+  *cap = bytes;
+  return DFS_OK;
+}
+void give_back_retired(dfs_ctx* c) {
+  for (void* p : c->retired) cudaFreeAsync(p, c->stream);
+  c->retired.clear();
 }
 
 int materialise(dfs_ctx* c, StoreRec& r) {
@@ -703,11 +724,8 @@ int run_window(dfs_ctx* c, const CachedWindow& cw, const WindowInfo& wi) {
     if (L.partial_bytes > c->partials_cap) {
       if (c->capturing)
         return fail(c, DFS_ERR_STATE, "reduction scratch would grow inside a capture: run the window once first");
-      if (c->partials) cudaFreeAsync(c->partials, c->stream);
-      c->partials = nullptr;
-      size_t cap = std::max<size_t>(L.partial_bytes, 4096);
-      CUDA_OK(cudaMallocAsync(&c->partials, cap, c->stream));
-      c->partials_cap = cap;
+      const int rc = grow_scratch(c, &c->partials, &c->partials_cap, std::max<size_t>(L.partial_bytes, 4096));
+      if (rc) return rc;
     }
     if (L.waves) {
       const int rc = reserve_flags(c);
@@ -1193,15 +1211,13 @@ int flush_batch(dfs_ctx* c) {
       release_window(c);
       return fail(c, DFS_ERR_STATE, "batch scratch would grow inside a capture: run the batch once before");
     }
-    if (sval_need > c->sval_cap) {
-      if (c->sval) cudaFreeAsync(c->sval, c->stream);
-      CUDA_OK(cudaMallocAsync((void**)&c->sval, sval_need, c->stream));
-      c->sval_cap = sval_need;
-    }
-    if (part_need > c->partials_cap) {
-      if (c->partials) cudaFreeAsync(c->partials, c->stream);
-      CUDA_OK(cudaMallocAsync(&c->partials, part_need, c->stream));
-      c->partials_cap = part_need;
+    void* sv = c->sval;
+    int rc = grow_scratch(c, &sv, &c->sval_cap, sval_need);
+    c->sval = (double*)sv;
+    if (!rc) rc = grow_scratch(c, &c->partials, &c->partials_cap, part_need);
+    if (rc) {
+      release_window(c);
+      return rc;
     }
   }
   // launch: struct BP { insts, prefix, sval, partials, ctl, timeout_ns, ninst, red_stride }
@@ -1512,6 +1528,7 @@ int dfs_shutdown(dfs_ctx* c) {
       if (c->partials) cudaFreeAsync(c->partials, c->stream);
       if (c->sval) cudaFreeAsync(c->sval, c->stream);
       if (c->flags) cudaFreeAsync(c->flags, c->stream);
+      give_back_retired(c);
       for (auto& kv : c->tables) cudaFreeAsync(kv.second.dev, c->stream);
       c->tables.clear();
       cudaStreamSynchronize(c->stream);
@@ -2066,12 +2083,8 @@ int dfs_capture_begin(dfs_ctx* c) {
     c->lastb.ok = false;
     // reduction scratch cannot be reallocated inside a capture: reserve 1 MB
     const size_t want = 1 << 20;
-    if (c->partials_cap < want) {
-      if (c->partials) cudaFreeAsync(c->partials, c->stream);
-      c->partials = nullptr;
-      CUDA_OK(cudaMallocAsync(&c->partials, want, c->stream));
-      c->partials_cap = want;
-    }
+    rc = grow_scratch(c, &c->partials, &c->partials_cap, want);
+    if (rc) return rc;
     rc = reserve_flags(c);
     if (rc) return rc;
     CUDA_OK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
@@ -2175,6 +2188,7 @@ int dfs_graph_destroy(dfs_ctx* c, dfs_graph h) {
     cudaGraphDestroy(it->second.graph);
     for (void* p : it->second.owned) cudaFreeAsync(p, c->stream);
     c->graphs.erase(it);
+    if (c->graphs.empty()) give_back_retired(c);
     return DFS_OK;
   } catch (const std::exception& e_) {
     return internal_error(c, e_.what());
