@@ -687,11 +687,21 @@ int Gen::users(int64_t root) const {
   return k;
 }
 // Nest n of group g reads an array that the last sweep before it used, and runs
-// backwards over it.  FP32 only: x + s with 3 y after a sum of x, 2^24 elements,
-// 59.5 -> 54.7 us, but FP64 131.7 -> 140.4 (2^23 63.7 -> 64.8, 2^25 264.6 ->
-// 259.0; FP64 sweeps are bound by their pipe and lose more by the addresses).
+// backwards over it: x + s with 3 y after a sum of x, 2^24 FP32 elements, 59.5 ->
+// 54.7 us.  FP64 sweeps are bound by their pipe and lose by the addresses once
+// their own arrays do not stay in L2 (2^24 elements 131.7 -> 140.4, 4M 39.4 ->
+// 40.7; 2M 26.4 -> 25.1, CG at 1337^2 743 -> 736 us per ten iterations).
 bool Gen::revisits(int g, const Nest& n) const {
-  if (space_arg(S.tasks[n.first]).dtype != DFS_F32) return false;
+  std::set<int64_t> arrays;
+  int64_t bytes = 0;
+  for (int i = n.first; i < n.last; ++i)
+    for (const Arg& a : S.tasks[i].args) {
+      if (a.imm || a.nd == 0 || R(a.root).temp || !arrays.insert(a.root).second) continue;
+      int64_t e = (int64_t)dtype_size(a.dtype);
+      for (int d = 0; d < a.nd; ++d) e *= R(a.root).shape[d];
+      bytes += e;
+    }
+  if (space_arg(S.tasks[n.first]).dtype != DFS_F32 && bytes > 96000000) return false;
   int h = g - 1;
   while (h >= 0 && S.groups[h].scalar) --h;
   if (h < 0) return false;
