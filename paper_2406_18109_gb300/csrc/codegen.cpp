@@ -1290,20 +1290,23 @@ double pair_ops(const LaunchSpec& S, int g) {
 // Two phases: a barrier and two flat sweeps; FP32 by L2 and HBM, FP64 by the
 // FP64 pipe, which a flat sweep keeps busy on all SMs.
 double phases_us(const LaunchSpec& S, double elems, int esz, double ops, int nd) {
-  if (esz == 4) return 6.0 + elems / 0.48e6;
+  if (esz == 4) return 6.5 + elems / (8.0 * elems > 96e6 ? 0.385e6 : 0.48e6);
   const double pipe = elems / S.sms * (0.00045 + 0.00027 * ops);
   return nd == 3 ? std::max(std::min(10.0, 6.0 + elems / 8192.0), 7.5 + pipe) : std::max(S.block >= 1024 ? 11.0 : 9.0, 5.5 + pipe);
 }
-// Bands: the CTA's flags, then a row of the band at a time.  FP32: a row costs
-// a round trip to L2, or what its vectors take.  FP64: the schedulers share the
+// Bands: the CTA's flags, then a row of the band (and the two next to it) at a
+// time.  FP32: a row costs a round trip to L2, or what its vectors take; columns
+// next to panels cost more.  FP64: the schedulers share the
 // FP64 units in such a way that a row costs as if part of the warps were
 // rounded up to eight (measured: 5, 6, 7, 8 warps 1.6, 1.7, 1.9, 2.0; 9, 10,
 // 12, 14, 16 warps 3.1, 3.3, 3.5, 3.8, 4.0 times what a warp per scheduler
 // should), whatever lanes are active: narrow rows waste it.
 double bands_us(const LaunchSpec& S, const MarchGeom& M, int esz, double ops) {
-  if (esz == 4)
-    return 4.0 + M.BR * std::max(0.22, 0.03 * ops * M.K * std::pow(S.block / 256.0, 0.6) * (1.0 + 0.05 * std::max(0, M.K - 6))) *
-                     (M.PN > 1 ? 1.3 : 1.0);
+  if (esz == 4) {
+    const double row = 0.03 * ops * M.K * std::pow(S.block / 256.0, 0.6) * (1.0 + 0.05 * std::max(0, M.K - 6));
+    const double trip = 0.23 * std::pow(S.block / 256.0, 0.3);
+    return 3.5 + (M.BR + 2) * std::max(trip, row) * (1.0 + 0.2 * std::min<int64_t>(M.PN - 1, 3));
+  }
   const int w = M.GT * M.G / 32 * std::max(1, S.min_blocks);
   const double busy = w <= 4 ? 1.1 : w / 8.0 + (w + 7) / 8;
   const double row = busy * M.K * (0.066 + 0.002 * ops) * ops * ((double)M.rows * M.cols * esz > 96e6 ? 1.12 : 1.0);
@@ -1515,7 +1518,8 @@ MarchGeom march_geometry(const LaunchSpec& S, int g) {
              (C.PN > 1 ? (C.BR + 2) * (int64_t)edges.size() * esz : 0);
     if (C.smem > limit || C.NB * C.PN > kWaveTilesMax) continue;
     const double us = bands_us(S, C, (int)esz, ops);
-    if (us >= best) continue;
+    // equal: fewer vectors per thread, unless that takes more panels
+    if (pick.ok ? us > best + 1e-6 || (us > best - 1e-6 && C.PN > pick.PN) : us >= best) continue;
     pick = C;
     pick.ok = true;
     best = us;
@@ -1624,12 +1628,12 @@ void Gen::emit_march(int g, int sweeps) {
     << "u + grp) * " << M.BR << ", " << M.rows << ") : " << M.rows << ", rz = min(ra + " << M.BR << ", " << M.rows << ");\n";
   o << in2 << "const bool act = ra < rz;\n";
   o << in2 << "const int pb = (int)(blockIdx.x % " << M.PN << "u) * " << M.PC << ";\n";
-  // The warp's number comes through a shuffle: with it written in place NVRTC
-  // 13.0 turned (threadIdx.x >> 5) * K + k, where only lane 31 gets there, K is
-  // a power of two and a CTA has several groups, into the address of K - 1
-  // elements further on.
+  // With several groups the warp's number comes through a shuffle: with it
+  // written in place NVRTC 13.0 turned (threadIdx.x >> 5) * K + k, where only lane
+  // 31 gets there and K is a power of two, into the address of K - 1 elements
+  // further on.
   o << in2 << "const int lane = threadIdx.x & 31, lw = q >> 5;\n";
-  o << in2 << "const int wid = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);\n";
+  o << in2 << "const int wid = " << (M.G > 1 ? "__shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0)" : "(int)(threadIdx.x >> 5)") << ";\n";
   // one warp's vectors k are consecutive; vectors past the row repeat its last
   for (int k = 0; k < K; ++k) {
     o << in2 << "const int c" << k << " = pb + " << k * M.GT << " + q;\n";
