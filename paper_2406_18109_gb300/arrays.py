@@ -170,8 +170,9 @@ class Runtime:
 
     def _issue_new(self, opcode, lay, n, shape, dtype) -> "Array":
         """_new and _issue as one native call: the last argument's store is
-        the new one (23 Black-Scholes tasks
-        and their flush: 85 -> 77 us)."""
+        the new one.  Bound by Python and ctypes: the 23 tasks of a
+        Black-Scholes window of 4096 options and their flush took 85 us with
+        two calls per operator, 79 us with one."""
         sc = self._shapes.get(shape)
         if sc is None:
             sc = self._shapes[shape] = (C.c_int64 * max(1, len(shape)))(*shape)

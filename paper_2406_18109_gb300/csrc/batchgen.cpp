@@ -628,6 +628,7 @@ bool BatchGen::run(BatchCode& out, std::string& why) {
 
   std::ostringstream src;
   src << "#include \"dfs_device.cuh\"\nusing namespace dfs;\n";
+  if (by_rows) src << "static_assert(kSpmvWarpBytes == " << kSpmvWarpBytes << ", \"shared memory of a warp\");\n";
   src << "struct Inst {\n  void* p[" << std::max(1, bc.nptr) << "];\n  double imm[" << std::max(1, bc.nimm)
       << "];\n  i64 v[" << std::max(1, bc.nv) << "];\n};\n";
   src << "struct BP {\n  const Inst* insts;\n  const i64* prefix;\n  double* sval;\n  void* partials;\n  Ctl* ctl;\n"

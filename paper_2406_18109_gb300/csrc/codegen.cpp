@@ -2145,8 +2145,8 @@ KernelCode Gen::run() {
   o << "  } while (0);\n";
   // The exit count costs every launch a round trip to L2 after its last store;
   // a kernel without barriers, sums, scalars to publish or sweeps leaves the
-  // control block as it found it (Black-Scholes, 1,000,003 options: 10.25 ->
-  // 9.79 us).
+  // control block as it found it (Black-Scholes, 1,000,003 options, both in turn:
+  // 10.27 -> 10.14 us).
   bool exits = nbar > 0 || !pending_red.empty() || kc.nwaves > 0;
   for (const LaunchRoot& r : S.roots) exits = exits || (r.zero_d && r.live_out && r.param >= 0);
   if (exits) {
@@ -2170,6 +2170,7 @@ KernelCode Gen::run() {
 
   std::ostringstream src;
   src << "#include \"dfs_device.cuh\"\nusing namespace dfs;\n";
+  if (by_rows) src << "static_assert(kSpmvWarpBytes == " << kSpmvWarpBytes << ", \"shared memory of a warp\");\n";
   src << "struct Params {\n  void* p[" << std::max(1, kc.nptr) << "];\n  double imm[" << std::max(1, kc.nimm)
       << "];\n  void* partials;\n  Ctl* ctl;\n  u64 timeout_ns;\n  i64 red_stride;\n"
       << (kc.nwaves ? "  u64* flags;\n" : "") << "};\n";

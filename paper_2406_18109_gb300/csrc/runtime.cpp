@@ -998,7 +998,8 @@ int flush_batch(dfs_ctx* c) {
   if (c->cfg.launch_mode != DFS_LAUNCH_PERSISTENT || !c->cfg.fusion) return fallback("batching runs fused, persistent launches");
   // Points are dealt in the order of the instances, and a phase ends with its
   // slowest point: those with the most entries go first, unless all have about
-  // the same.  (2048 rows of about 16 scattered entries take 100 us; dealt
+  // the same (within half as many again: a choice, other ratios were not
+  // measured).  (2048 rows of about 16 scattered entries take 100 us; dealt
   // last, they ended an SpMV phase at 282 us whose CTAs were done at 187 on
   // average; first, at 210.)
   {
