@@ -512,11 +512,12 @@ class Arm:
         self.units = cfg["sweeps"]
         self.step = self._jacobi
         if self.autotune:
-            # rows per point and launch shape of the sweep
+            # launch shape of the sweep (an in-place sweep depends neither on
+            # the rows per point nor on the unroll factor)
             def sweep():
                 W.jacobi_sweep(self.views)
                 rt.flush()
-            self._tune(sweep, {"rows": [8, 16, 32], "block": [256, 512], "unroll": [4, 8], "ctas_per_sm": [0, 4, 6]},
+            self._tune(sweep, {"block": [256, 512], "ctas_per_sm": [0, 2]},
                        f"jacobi-{cfg['N']}", 3, "ms_per_sweep")
         if self.graph_mode:
             # the step's sweeps (one window per sweep, memoised) issued once,
@@ -936,7 +937,9 @@ def measure(args, workload, env, steps, warmup, cpu_budget=(10.0, 8.0)) -> dict:
         # iteration (12 for the FP64 count of the single-solve CG line)
         alg_bytes = (esz + 4) * nnz + 4 * (rows + cfg["count"]) + 12 * esz * rows
     else:
-        alg_bytes = 16 * cfg["N"] * cfg["N"]               # one sweep (one launch)
+        # one sweep (one launch), in place: every point read once and written
+        # once (the two phases of before moved twice that)
+        alg_bytes = 8 * cfg["N"] * cfg["N"]
     kern_ms = fused["dominant_ms"]
     if graph:
         # launches replayed from a graph are not timed one by one: use the
