@@ -12,8 +12,8 @@ BLACK_SCHOLES = dict(n=1 << 26, seed=1, r=0.02, sigma=0.3, tile=16384, block=102
                      # thread instructions per option (smsp__inst_executed x 32
                      # / options; the kernel is bound by instruction issue) and
                      # DRAM bytes (read + write) of one launch at n = 2^26
-                     counters=dict(kernel="dfs_k62b33cd1f6ebfe5d", inst_per_option=111.91,
-                                   dram_bytes_per_launch=1301.96e6),
+                     counters=dict(kernel="dfs_k38867f1183cfbff1", inst_per_option=111.48,
+                                   dram_bytes_per_launch=1301.88e6),
                      # end to end (host arrays): kernels on mapped host memory
                      # ("zero_copy") or copies pipelined in chunks over contexts
                      e2e_mode="zero_copy", e2e_chunk=1 << 23, e2e_contexts=2)
@@ -25,7 +25,7 @@ CG = dict(m=256, iters=50, seed=0, tile=512, block=256, unroll=1, iters_per_flus
           # ncu counters of the steady five-iteration window kernel named
           # `kernel` (this launch shape): DRAM bytes per iteration; the rest of
           # the traffic is served by L2 (profiles/)
-          counters=dict(kernel="dfs_kd2a6167401cf8ba5", dram_bytes_per_iteration=5.851904e6 / 5))
+          counters=dict(kernel="dfs_kdd08d9c86138047a", dram_bytes_per_iteration=5.852416e6 / 5))
 
 # Batched CG: 256 independent solves of uneven size (half 2-D Poisson with m
 # log-uniform in [32, 1024], half random diagonally dominant SPD with n
@@ -38,15 +38,15 @@ BATCHED_CG = dict(count=256, seed=4, iters=100, dtype="f64", tile_max=2048, min_
                   # ncu counters of the batched iteration kernel named `kernel`,
                   # FP64 and FP32, at this launch shape: DRAM bytes (read + write)
                   # per launch (profiles/)
-                  counters=[dict(kernel="dfs_b0fc715b3e5f18a2c", dram_bytes_per_launch=3.019141e9 + 0.672542e9),
-                            dict(kernel="dfs_b0a54bf6785d3c28c", dram_bytes_per_launch=1.865591e9 + 0.315713e9)])
+                  counters=[dict(kernel="dfs_b2605c33e74bf8cdd", dram_bytes_per_launch=3.009157e9 + 0.673192e9),
+                            dict(kernel="dfs_bd7c824ace6e25847", dram_bytes_per_launch=1.804926e9 + 0.315192e9)])
 
 # Jacobi: Fig. 1 stencil on an 8192x8192 FP32 grid (8190^2 interior),
 # 200 sweeps, interior U[0,1] (seed 2), boundary 1.0
 JACOBI = dict(N=8190, sweeps=200, seed=2, rows=16, block=512, unroll=4, sweeps_per_flush=1,
               # ncu counters (one-pass metrics, full size) of the sweep kernel
               # named `kernel`: DRAM bytes (read + write) of one launch (one sweep)
-              counters=dict(kernel="dfs_ka23239f399de85c0", dram_bytes_per_launch=540.48e6 + 487.56e6))
+              counters=dict(kernel="dfs_k4cefc98c08d22dd7", dram_bytes_per_launch=273.43e6 + 206.36e6))
 
 # Serving: Poisson arrivals (exponential gaps, mean 2 ms, seed 3) of CG and
 # BiCGSTAB solves on 3-D 7-point Poisson operators (m from a log-spaced

@@ -1212,7 +1212,7 @@ int Gen::emit_warp0_scalars(int g) {
 // per FP32 point and is bound by HBM; in place it is 8.  Measured on GB300, us
 // per sweep, two phases -> in place:
 //   8190^2 FP32 (512-thread CTAs)        175.6 -> 91.9 (5.84 TB/s, 86 % of the copy rate)
-//   1021 x 1147 FP32, five per launch      8.3 -> 4.4
+//   1021 x 1147 FP32, five per launch      7.9 -> 4.3
 //   4000^2 FP64                          197.4 -> 174.4 (bound by the FP64 pipe: 5 operations per point)
 //   251^3 FP32 (tiles)                    64.1 -> 42.1
 //   251^3 FP64 (tiles)                   258.9 -> 242 (FP64 pipe: 7 operations per point, 176 us)
